@@ -1,6 +1,6 @@
 """Build the solver library ``libhs.so`` in-tree with nvcc for sm_103a.
 
-The four translation units compile in parallel; objects go to
+The translation units compile in parallel; objects go to
 ``paper_2405_11168_gb300/_build/`` (git-ignored) and the shared library to
 ``paper_2405_11168_gb300/libhs.so``.  The CUDA runtime is linked statically,
 so the library loads without a GPU (only kernel launches need one).
@@ -17,7 +17,8 @@ SRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhs.so")
 UNITS = ["capi.cu", "kernels_util.cu", "kernels_f32.cu", "kernels_f64.cu", "kernels_ext_f32.cu",
-         "kernels_ext_f64.cu", "noalloc.cu"]
+         "kernels_ext_f64.cu", "kernels_real_iso_f32.cu", "kernels_real_aniso_f32.cu",
+         "kernels_real_iso_f64.cu", "kernels_real_aniso_f64.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

@@ -21,6 +21,7 @@
 
 #include "../../include/hs.h"
 #include "launch.h"
+#include "tiling.h"
 
 using hs::DevStatus;
 using hs::FftPlan;
@@ -31,9 +32,7 @@ thread_local std::string g_last_error;
 
 constexpr int kHistCap = 1 << 16;
 constexpr int kMaxN = 512;
-// Real-space pass blocks: ~7 per SM (z chunks of 16 planes at 256^3).  Longer
-// chunks re-read fewer halo planes; measured on GB300 at 256^3 (TY = 4):
-// 0.327 / 0.283 / 0.266 / 0.261 / 0.270 / 0.280 ms for chunks of 4 / 8 / 12 / 16 / 24 / 32.
+// Blocks of the fused x pass (xfuse = 1): ~7 per SM.
 constexpr int kTargetBlocks = 1024;
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -501,42 +500,20 @@ int pitch_of(int nh, bool f64) { return f64 ? ((nh + 1) & ~1) : ((nh + 3) & ~3);
 
 int pick_ty(int n2) { return (n2 % 4 == 0) ? 4 : 2; }
 
-// z chunk of an FP64 real-space pass.  Its blocks (one per (y tile, z chunk), launched y tile
-// first) are bound by the FP64 pipe, so a block's time is proportional to the voxel layers it
-// computes (chunk + 1) and the pass ends when a greedy list schedule of the blocks, in launch
-// order, on the resident slots ends.  The chunk length with the earliest end is taken (the longer
-// on ties: fewer recomputed layers).  At 256^3 on GB300 this model reproduces the measured
-// sweep times of chunks 8..32 to 1%.
-int pick_zchunk64(int yt, int n3, int slots) {
-  int best_zc = 0;
-  long long best = -1;
-  std::vector<long long> heap(std::max(slots, 1));
-  for (int zc = std::min(4, n3); zc <= std::min(n3, 64); ++zc) {
-    std::fill(heap.begin(), heap.end(), 0LL);
-    long long end = 0;
-    const int nz = (n3 + zc - 1) / zc;
-    for (int z = 0; z < nz; ++z) {
-      const long long layers = std::min(zc, n3 - z * zc) + 1;
-      for (int y = 0; y < yt; ++y) {
-        std::pop_heap(heap.begin(), heap.end(), std::greater<long long>());
-        heap.back() += layers;
-        end = std::max(end, heap.back());
-        std::push_heap(heap.begin(), heap.end(), std::greater<long long>());
-      }
-    }
-    if (best < 0 || end < best || (end == best && zc > best_zc)) {
-      best = end;
-      best_zc = zc;
-    }
-  }
-  return best_zc;
+size_t march_smem(int n1, int ty, bool f64, int mode, bool real, bool has_src = false) {
+  const int nthr = ((n1 + 31) / 32) * 32, ts = f64 ? 8 : 4;
+  if (real) return hs::real_layout(hs::real_pitch(f64, ty, mode, n1), nthr, ty, has_src, ts).total;
+  return hs::march_layout(n1, pitch_of(n1 / 2 + 1, f64), nthr, ty, mode, has_src, ts).total;
 }
 
-size_t march_smem(int n1, int ty, bool f64, int mode, bool real, bool has_src = false) {
-  const int nh = n1 / 2 + 1;
-  const int P = real ? 0 : pitch_of(nh, f64);
-  const int nthr = ((n1 + 31) / 32) * 32;
-  return hs::march_layout(n1, P, nthr, ty, mode, real, has_src, f64 ? 8 : 4).total;
+// Largest shared memory of a real-space tile that an explicit ytile may ask for: the planes, two source
+// buffers, ids and edges of the tile.  (The pass itself keeps a third source buffer; a tile that only
+// just fits runs with half its rows.)
+size_t real_tile_bytes(int n1, int ty, bool f64) {
+  const size_t ts = f64 ? 8 : 4, nw = (n1 + 31) / 32, nr = ty + 2;
+  auto al = [](size_t x) { return hs::hs_align16(x); };
+  return al(ts * 9 * nr * n1) + al((size_t)4 * (ty + 1) * ((n1 + 7) & ~7)) + al((size_t)24 * ty * ((n1 + 3) & ~3)) +
+         al(ts * nw * (ty + 1) * 12) + 1824;
 }
 
 Layout make_layout(int n1, int n2, int n3, int nphase, int prec) {
@@ -553,10 +530,10 @@ Layout make_layout(int n1, int n2, int n3, int nphase, int prec) {
   L.B1 = off; off += cbuf;
   L.F = off; off += cbuf;
   L.ids = off; off += align256(N * 2);
-  L.matk = off; off += align256((size_t)nphase * 21 * (f64 ? 8 : 4));
-  L.matd = off; off += align256((size_t)nphase * 21 * 8);
+  L.matk = off; off += align256((size_t)nphase * (f64 ? hs::kAnisoStride<double> * 8 : hs::kAnisoStride<float> * 4));
+  L.matd = off; off += align256((size_t)nphase * hs::kAnisoStride<double> * 8);
   L.tw = off; off += align256((size_t)(n1 + n2 + n3) * cs);
-  L.partials = off; off += align256(max_blocks * hs::NRED * 8);
+  L.partials = off; off += align256(max_blocks * hs::kPartStride * 8);
   L.status = off; off += align256(sizeof(DevStatus));
   L.hist = off; off += align256((size_t)kHistCap * 8);
   L.macro = off; off += align256(42 * 8);
@@ -592,6 +569,13 @@ template <typename T> void fill_march_common(hs_ctx* c, hs::MarchArgs<T>& a) {
   a.st = c->st;
   a.hist = c->hist;
   a.zstride = c->batch_stride;
+}
+
+// rows of k_real: their shared-memory pitch, and bulk copies where every row starts and ends on 16 bytes
+// (the workspace buffers are 256-byte aligned)
+template <typename T> void set_real_rows(hs::MarchArgs<T>& a, int ty, int mode) {
+  a.xp = hs::real_pitch(sizeof(T) == 8, ty, mode, a.n1);
+  a.bulk = (a.n1 % 8 == 0) ? 1 : 0;
 }
 
 template <typename T> void fill_col(hs_ctx* c, hs::ColArgs<T>& a, void* buf, int axis) {
@@ -637,7 +621,7 @@ template <typename T> hs_status launch_force(hs_ctx* c, const double E[6], int i
   a.skip_if_done = 1;
   const size_t sm = march_smem(c->n1, c->ty, sizeof(T) == 8, hs::MODE_FORCE, false, src != nullptr);
   LaunchScope ls(c, HS_K_XPASS);
-  cudaError_t e = hs::launch_march<T>(a, c->iso, c->ty, hs::MODE_FORCE, false, c->grid_m, c->nthr_m, sm, c->stream);
+  cudaError_t e = hs::launch_march<T>(a, c->iso, c->ty, hs::MODE_FORCE, c->grid_m, c->nthr_m, sm, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "k_march(force)");
   return HS_OK;
 }
@@ -659,6 +643,11 @@ template <typename T> hs_status launch_rows(hs_ctx* c, int mode, double* acc64, 
   a.st = c->st;
   a.skip_if_done = skip ? 1 : 0;
   a.zstride = c->batch_stride;
+  if (mode == hs::ROW_R2C) {  // this pass takes the stopping test of the evaluation before it
+    a.partials = c->partials;
+    a.nparts = (int)(c->grid_m.x * c->grid_m.y);
+    a.hist = c->hist;
+  }
   cudaError_t e;
   {
     LaunchScope ls(c, acc64 ? HS_K_OTHER : (mode == hs::ROW_C2R ? HS_K_XINV : HS_K_XFWD));
@@ -689,13 +678,15 @@ template <typename T> hs_status launch_stencil(hs_ctx* c, const double E[6], con
   a.sig_out = sig;
   a.out_f32 = c->opt.out_f32;
   a.skip_if_done = (mode == hs::MODE_FORCE) ? 1 : 0;
+  set_real_rows(a, c->ty, mode);
+  a.defer = (mode == hs::MODE_FORCE) ? 1 : 0;  // the forward row pass follows
   const size_t sm = march_smem(c->n1, c->ty, sizeof(T) == 8, mode, true, src != nullptr);
   cudaError_t e;
   {
     LaunchScope ls(c, mode == hs::MODE_FORCE ? (src != nullptr ? HS_K_XPASS_SRC : HS_K_XPASS) : HS_K_FIELDS);
-    e = hs::launch_march<T>(a, c->iso, c->ty, mode, true, zg(c, c->grid_m), c->nthr_m, sm, c->stream);
+    e = hs::launch_real<T>(a, c->iso, c->ty, mode, zg(c, c->grid_m), c->nthr_m, sm, c->stream);
   }
-  if (e != cudaSuccess) return cuda_fail(c, e, "k_march(real)");
+  if (e != cudaSuccess) return cuda_fail(c, e, "k_real");
   return HS_OK;
 }
 
@@ -827,7 +818,7 @@ template <typename T> hs_status launch_fields(hs_ctx* c, const double E[6], int 
   a.skip_if_done = 0;
   const size_t sm = march_smem(c->n1, c->ty, sizeof(T) == 8, hs::MODE_FIELDS, false);
   LaunchScope ls(c, HS_K_FIELDS);
-  cudaError_t e = hs::launch_march<T>(a, c->iso, c->ty, hs::MODE_FIELDS, false, c->grid_m, c->nthr_m, sm, c->stream);
+  cudaError_t e = hs::launch_march<T>(a, c->iso, c->ty, hs::MODE_FIELDS, c->grid_m, c->nthr_m, sm, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "k_march(fields)");
   return HS_OK;
 }
@@ -978,8 +969,8 @@ hs_status solve_plain(hs_ctx* c, const double E[6], double tol, int max_iter, vo
     if (c->xfuse) {
       s = launch_fields<T>(c, E, last_in, eps, sig);
     } else {
-      s = launch_rows<T>(c, hs::ROW_C2R, nullptr, false);
-      if (s == HS_OK) s = launch_stencil<T>(c, E, nullptr, hs::MODE_FIELDS, eps, sig);
+      // B[1] still holds the displacement of the last evaluation (every later kernel was skipped)
+      s = launch_stencil<T>(c, E, nullptr, hs::MODE_FIELDS, eps, sig);
     }
     if (s != HS_OK) return s;
   }
@@ -1004,14 +995,15 @@ hs_status launch_residual64(hs_ctx* c, const double E[6], int mode, void* eps, v
   a.fout = c->rsrc;
   a.fout_f32 = 1;
   a.zc = c->zc64;
+  set_real_rows(a, c->ty64, mode);
   a.eps_out = eps;
   a.sig_out = sig;
   a.out_f32 = c->opt.out_f32;
   a.skip_if_done = 0;
   const size_t sm = march_smem(c->n1, c->ty64, true, mode, true);
   LaunchScope ls(c, mode == hs::MODE_FIELDS ? HS_K_FIELDS : HS_K_RESID64);
-  cudaError_t e = hs::launch_march<double>(a, c->iso, c->ty64, mode, true, zg(c, c->grid_m64), c->nthr_m, sm, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "k_march(residual fp64)");
+  cudaError_t e = hs::launch_real<double>(a, c->iso, c->ty64, mode, zg(c, c->grid_m64), c->nthr_m, sm, c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "k_real(residual fp64)");
   return HS_OK;
 }
 
@@ -1023,7 +1015,7 @@ hs_status launch_emit(hs_ctx* c, int in) {
   a.skip_if_done = 0;
   const size_t sm = march_smem(c->n1, c->ty, false, hs::MODE_EMIT, false);
   LaunchScope ls(c, HS_K_OTHER);
-  cudaError_t e = hs::launch_march<float>(a, true, c->ty, hs::MODE_EMIT, false, c->grid_m, c->nthr_m, sm, c->stream);
+  cudaError_t e = hs::launch_march<float>(a, true, c->ty, hs::MODE_EMIT, c->grid_m, c->nthr_m, sm, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "k_march(emit)");
   return HS_OK;
 }
@@ -1431,67 +1423,49 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
     delete c;
     return st;
   }
-  // real-space pass: an automatic row tile is halved while its plane ring does not fit
-  // (FP64 rows of 512 need 2 rows per block)
-  if (o.ytile == 0 && !c->xfuse) {
-    int ty = c->ty;
-    while (ty > 2 && march_smem(c->n1, ty, c->f64, hs::MODE_FORCE, true, true) > (size_t)smem_optin) ty /= 2;
-    if (ty != c->ty && c->n2 % ty == 0) {
-      c->ty = ty;
-      const int yt = c->n2 / c->ty;
-      int nz = std::max(1, std::min(c->n3, (kTargetBlocks + yt - 1) / yt));
-      c->zc = (c->n3 + nz - 1) / nz;
-      if (o.zchunk > 0) c->zc = std::min(o.zchunk, c->n3);
-      nz = (c->n3 + c->zc - 1) / c->zc;
-      c->grid_m = dim3(yt, nz);
+  // real-space pass on a real displacement: row tile and z chunk
+  int nsm = 1;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int nwarps = c->nthr_m / 32;
+  auto real_smem = [&](int ty, bool f64, bool src) { return march_smem(c->n1, ty, f64, hs::MODE_FORCE, true, src); };
+  auto tile_fits = [&](int ty, bool f64) { return real_smem(ty, f64, !f64) <= (size_t)smem_optin; };
+  auto pick64 = [&](int fixed_ty, int fixed_zc, int* ty, int* zc) {
+    hs::pick_tile64(c->iso, c->n1, c->n2, c->n3, fixed_ty, (size_t)smem_optin, std::max(1, nsm), 0, ty, zc);
+    if (fixed_zc > 0) *zc = std::min(fixed_zc, c->n3);
+  };
+  int ytile = o.ytile;
+  if (!c->xfuse) {
+    if (ytile > 0 && real_tile_bytes(c->n1, ytile, c->f64) > (size_t)smem_optin) {
+      delete c;
+      return fail(nullptr, HS_ERR_UNSUPPORTED_SIZE, "grid too large for shared-memory tiles");
     }
-  }
-  // FP64 precision: the real-space pass is FP64-bound like the refined mode's sweep
-  if (c->f64 && !c->xfuse && o.zchunk == 0) {
-    int per_sm = 0, nsm = 0;
-    const size_t smf = march_smem(c->n1, c->ty, true, hs::MODE_FORCE, true);
-    if (hs::march_blocks_per_sm<double>(c->iso, c->ty, c->nthr_m, smf, &per_sm) == cudaSuccess &&
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && per_sm > 0) {
-      const int yt = c->n2 / c->ty;
-      c->zc = pick_zchunk64(yt, c->n3, per_sm * nsm);
-      c->grid_m = dim3(yt, (c->n3 + c->zc - 1) / c->zc);
+    while (ytile > 2 && !tile_fits(ytile, c->f64)) ytile /= 2;
+    if (c->f64) {
+      pick64(ytile, o.zchunk, &c->ty, &c->zc);
     } else {
-      cudaGetLastError();
+      if (ytile > 0) c->ty = ytile;
+      while (c->ty > 2 && !tile_fits(c->ty, false)) c->ty /= 2;
+      const int occ = hs::real_occupancy<float>(c->iso, c->n1, c->ty, real_smem(c->ty, false, o.precision == HS_FP32_REFINED));
+      c->zc = o.zchunk > 0 ? std::min(o.zchunk, c->n3)
+                           : hs::pick_zchunk32(c->n2 / c->ty, c->n3, nwarps, std::max(1, occ), std::max(1, nsm));
     }
+    c->grid_m = dim3(c->n2 / c->ty, (c->n3 + c->zc - 1) / c->zc);
   }
-  // FP64 residual sweep: the widest row tile whose plane ring fits; 8 rows (1/8 of the rows
-  // recomputed, not 1/4, and no register spills in blocks of at most 256 threads) where N1 <= 256
   c->ty64 = c->ty;
+  c->zc64 = c->zc;
   if (o.precision == HS_FP32_REFINED) {
-    if (o.ytile == 0 && c->n1 <= 256 && c->n2 % 8 == 0 &&
-        march_smem(c->n1, 8, true, hs::MODE_FORCE, true) <= (size_t)smem_optin)
-      c->ty64 = 8;
-    while (c->ty64 > 2 && march_smem(c->n1, c->ty64, true, hs::MODE_FORCE, true) > (size_t)smem_optin) c->ty64 /= 2;
-    if (c->n2 % c->ty64 != 0) c->ty64 = 2;
+    int t = ytile;  // the FP64 sweep's tile follows an explicit ytile, halved while it does not fit
+    while (t > 2 && !tile_fits(t, true)) t /= 2;
+    pick64(t, 0, &c->ty64, &c->zc64);
   }
-  {
-    const int yt = c->n2 / c->ty64;
-    int nz = std::max(1, std::min(c->n3, (kTargetBlocks + yt - 1) / yt));
-    c->zc64 = (c->n3 + nz - 1) / nz;
-    if (o.precision == HS_FP32_REFINED) {
-      int per_sm = 0, nsm = 0;
-      const size_t sm64 = march_smem(c->n1, c->ty64, true, hs::MODE_FORCE, true);
-      if (hs::march_blocks_per_sm<double>(c->iso, c->ty64, c->nthr_m, sm64, &per_sm) == cudaSuccess &&
-          cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && per_sm > 0)
-        c->zc64 = pick_zchunk64(yt, c->n3, per_sm * nsm);
-      else
-        cudaGetLastError();
-    }
-    nz = (c->n3 + c->zc64 - 1) / c->zc64;
-    c->grid_m64 = dim3(yt, nz);
-  }
+  c->grid_m64 = dim3(c->n2 / c->ty64, (c->n3 + c->zc64 - 1) / c->zc64);
   // z pass: the state tile in shared memory beside the force tile when asked for (col_state = 2)
   if (o.col_state == 2 && 2 * c->smem_z <= (size_t)smem_optin) {
     c->zstate_smem = true;
     c->smem_z *= 2;
   }
   const size_t need = std::max({c->xfuse ? march_smem(c->n1, c->ty, c->f64, hs::MODE_FORCE, false, true)
-                                          : march_smem(c->n1, c->ty, c->f64, hs::MODE_FORCE, true, true),
+                                          : march_smem(c->n1, c->ty, c->f64, hs::MODE_FORCE, true, !c->f64),
                                 c->smem_row[0], c->smem_row[1],
                                 o.precision == HS_FP32_REFINED ? march_smem(c->n1, c->ty64, true, hs::MODE_FORCE, true) : 0,
                                 c->smem_y, c->smem_z});
@@ -1501,7 +1475,6 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
   }
   // persistent row passes: as many blocks as stay resident, at most one per batch
   {
-    int nsm = 0;
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int T8 = (c->n1 + hs::kE - 1) / hs::kE;
     const size_t G = (size_t)(c->nthr_row / T8);
@@ -1511,6 +1484,9 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
       e = c->f64 ? hs::row_blocks_per_sm<double>(m, c->n1, c->nthr_row, c->smem_row[m], &per_sm)
                  : hs::row_blocks_per_sm<float>(m, c->n1, c->nthr_row, c->smem_row[m], &per_sm);
       c->nblk_row[m] = (int)std::min<size_t>(nbatch, (size_t)std::max(1, per_sm) * std::max(1, nsm));
+      // the forward pass gives one of its resident blocks to the stopping test
+      if (m == hs::ROW_R2C)
+        c->nblk_row[m] = 1 + (int)std::min<size_t>(nbatch, (size_t)std::max(1, per_sm * std::max(1, nsm) - 1));
     }
     if (e != cudaSuccess) {
       hs_status st = cuda_fail(nullptr, e, "row pass occupancy");
@@ -1521,8 +1497,6 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
 
   // persistent double-buffered y / z passes at the compile-time lengths (default tile and block)
   {
-    int nsm = 0;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const bool ext = hs::plan_ext(c->plan[1]) || hs::plan_ext(c->plan[2]);
     const int xtiles = (c->nh + c->ct - 1) / c->ct;
     // the z pass stays one tile per block: its Green step waits on the state point by point, and
@@ -1590,16 +1564,20 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
       delete c;
       return st;
     }
-    std::vector<double> md((size_t)np * 21);
+    // phase tables in the kernels' layouts (common.cuh)
+    std::vector<double> md((size_t)np * hs::kAnisoStride<double>, 0.0);
+    std::vector<float> mf(c->f64 ? 0 : (size_t)np * hs::kAnisoStride<float>, 0.f);
     for (int p = 0; p < np; ++p) {
-      const double* C = &table[(size_t)p * 36];
       if (all_iso) {
-        md[(size_t)p * 2] = lam[p];
-        md[(size_t)p * 2 + 1] = mu[p];
+        hs::pack_iso(lam[p], mu[p], &md[(size_t)p * hs::kIsoStride<double>]);
       } else {
-        int k = 0;
-        for (int i = 0; i < 6; ++i)
-          for (int j = i; j < 6; ++j) md[(size_t)p * 21 + k++] = C[i * 6 + j];
+        hs::pack_upper(&table[(size_t)p * 36], &md[(size_t)p * hs::kAnisoStride<double>]);
+      }
+      if (c->f64) continue;
+      if (all_iso) {
+        hs::pack_iso(lam[p], mu[p], &mf[(size_t)p * hs::kIsoStride<float>]);
+      } else {
+        hs::pack_upper(&table[(size_t)p * 36], &mf[(size_t)p * hs::kAnisoStride<float>]);
       }
     }
     {
@@ -1619,7 +1597,6 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
       if (c->f64) {
         e = cudaMemcpyAsync(c->matk, md.data(), md.size() * 8, cudaMemcpyHostToDevice, c->stream);
       } else {
-        std::vector<float> mf(md.begin(), md.end());
         e = cudaMemcpyAsync(c->matk, mf.data(), mf.size() * 4, cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
       }

@@ -50,12 +50,34 @@ template <typename P> __device__ __forceinline__ P* zshift(P* p, size_t off) {
   return p == nullptr ? p : reinterpret_cast<P*>(reinterpret_cast<uintptr_t>(p) + off);
 }
 constexpr int NRED = 7;  // sum of sigma^T1 + sigma^T2 (6), sum |F|^2 (1)
+constexpr int kPartStride = 8;                       // a block's partial sums in memory: NRED values, one spare
+constexpr size_t kReduceScratch = 32 * kPartStride * 8;  // shared memory of reduce_and_finalize
 
-// Isotropic phases: per phase (lambda, mu).
+// Phase tables.  Isotropic phases: FP32 (lambda, lambda, mu, mu), one 16-byte load of the pairs that
+// the two-lane arithmetic takes; FP64 (lambda, mu).  Anisotropic phases: the 21 upper-triangle entries
+// of the 6x6 Voigt stiffness, row-major, padded to whole 16-byte loads.
+// The stored stiffness is kTabScale times the material's (a power of two; see real.cuh).
+template <typename T> constexpr T kTabScale = T(0.0625);
+template <typename T> constexpr int kIsoStride = sizeof(T) == 4 ? 4 : 2;
+template <typename T> constexpr int kAnisoStride = sizeof(T) == 4 ? 24 : 22;
+__device__ __forceinline__ void iso_pairs(const float* tab, int ph, float2& lam, float2& mu) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(tab) + ph);
+  lam = make_float2(v.x, v.y);
+  mu = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void iso_pairs(const double* tab, int ph, double2& lam, double2& mu) {
+  const double2 v = __ldg(reinterpret_cast<const double2*>(tab) + ph);
+  lam = make_double2(v.x, v.x);
+  mu = make_double2(v.y, v.y);
+}
+
+// Isotropic phases.
 template <typename T> struct MatIso {
   const T* tab;
   __device__ __forceinline__ void stress(int ph, const T* e, T* s) const {
-    const T lam = __ldg(tab + 2 * ph), mu = __ldg(tab + 2 * ph + 1);
+    typename cplx_t<T>::type lp, mp;
+    iso_pairs(tab, ph, lp, mp);
+    const T lam = lp.x / kTabScale<T>, mu = mp.x / kTabScale<T>;
     const T lt = lam * (e[0] + e[1] + e[2]);
     const T m2 = mu + mu;
     s[0] = lt + m2 * e[0];
@@ -67,15 +89,14 @@ template <typename T> struct MatIso {
   }
 };
 
-// General anisotropic phases: per phase the 21 upper-triangle entries of the
-// 6x6 Voigt stiffness, row-major.  e is the engineering Voigt strain.
+// General anisotropic phases.  e is the engineering Voigt strain.
 template <typename T> struct MatAniso {
   const T* tab;
   __device__ __forceinline__ void stress(int ph, const T* e, T* s) const {
-    const T* c = tab + 21 * ph;
+    const T* c = tab + kAnisoStride<T> * ph;
     T C[21];
 #pragma unroll
-    for (int i = 0; i < 21; ++i) C[i] = __ldg(c + i);
+    for (int i = 0; i < 21; ++i) C[i] = __ldg(c + i) / kTabScale<T>;
     // index of (i,j), i <= j, in the packed upper triangle
 #define HS_UT(i, j) ((i) * 6 - ((i) * ((i) - 1)) / 2 + ((j) - (i)))
 #pragma unroll
@@ -89,23 +110,21 @@ template <typename T> struct MatAniso {
   }
 };
 
-template <typename T> __device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Evaluation of the stopping test from the sums of one residual evaluation
 // (Eqs. L2-norm, tolerance): sums[0..5] = sum over voxels of sigma^T1 + sigma^T2,
 // sums[6] = sum over corners of |F|^2.  Updates the status (error, history,
 // done flag, applied-stress strain update) and clears the arrival counter.
-// One thread calls it.
+// One thread calls it.  The status is read in one go, past L1 (other blocks of
+// this launch may have recorded a timeout in it).
 __device__ inline void finalize_eval(DevStatus* st, double* hist, const double* sums) {
-  if (st->done == DONE_TIMEOUT || st->done == DONE_FAULT) {
-    st->counter = 0;
-    return;
-  }
-  const double n = st->nvox;
+  const int done0 = __ldcg(&st->done), k = __ldcg(&st->evals), max_iter = __ldcg(&st->max_iter),
+            hist_cap = __ldcg(&st->hist_cap);
+  const double tol = __ldcg(&st->tol), denom = __ldcg(&st->denom), n = __ldcg(&st->nvox),
+               rel_tol = __ldcg(&st->rel_tol), err_min0 = __ldcg(&st->err_min), err_first0 = __ldcg(&st->err_first);
+  const double* const macro =
+      reinterpret_cast<const double*>(__ldcg(reinterpret_cast<const unsigned long long*>(&st->macro)));
+  st->counter = 0;
+  if (done0 == DONE_TIMEOUT || done0 == DONE_FAULT) return;
   double sm[6], nrm2 = 0;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
@@ -115,30 +134,33 @@ __device__ inline void finalize_eval(DevStatus* st, double* hist, const double* 
   }
   const double l2 = sqrt(sums[6] / n);
   const double nrm = sqrt(nrm2);
-  const double den = st->denom > 0 ? st->denom : nrm;
+  const double den = denom > 0 ? denom : nrm;
   double err;
   if (den > 0) err = l2 / den;
   else err = (l2 == 0) ? 0.0 : __longlong_as_double(0x7ff0000000000000LL);
   st->l2 = l2;
   st->sig_norm = nrm;
   st->err = err;
-  const int k = st->evals;
-  if (k < st->hist_cap) hist[k] = err;
+  if (k < hist_cap) hist[k] = err;
   st->evals = k + 1;
+  int done = DONE_RUNNING;
   if (!(err == err) || err > 1e300) {
-    st->done = DONE_DIVERGED;
+    done = DONE_DIVERGED;
   } else {
-    if (k == 0 || err < st->err_min) st->err_min = err;
-    if (k == 0) st->err_first = err;
-    if (err < st->tol || (st->rel_tol > 0 && err <= st->rel_tol * st->err_first)) st->done = DONE_CONVERGED;
-    else if (err > 1e6 * st->err_min && k > 10) st->done = DONE_DIVERGED;
-    else if (k + 1 >= st->max_iter) st->done = DONE_MAXITER;
+    const double err_min = (k == 0 || err < err_min0) ? err : err_min0;
+    const double err_first = k == 0 ? err : err_first0;
+    st->err_min = err_min;
+    st->err_first = err_first;
+    if (err < tol || (rel_tol > 0 && err <= rel_tol * err_first)) done = DONE_CONVERGED;
+    else if (err > 1e6 * err_min && k > 10) done = DONE_DIVERGED;
+    else if (k + 1 >= max_iter) done = DONE_MAXITER;
   }
-  if (st->macro != nullptr && st->done == DONE_RUNNING) {
+  if (done != DONE_RUNNING) atomicMax(&st->done, done);  // a timeout recorded meanwhile stays
+  if (macro != nullptr && done == DONE_RUNNING) {
     // E <- (lambda0)^-1 : {sigma^a + (lambda0 - <lambda>) : E - <lambda : deps> + <lambda : eps0>}
     //    = E + (lambda0)^-1 : (sigma^a - <sigma>)   (the same quantity, regrouped)
-    const double* Sa = st->macro;
-    const double* S0 = st->macro + 6;
+    const double* Sa = macro;
+    const double* S0 = macro + 6;
     double d[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) d[i] = Sa[i] - sm[i];
@@ -150,25 +172,46 @@ __device__ inline void finalize_eval(DevStatus* st, double* hist, const double* 
       st->E[i] += acc;
     }
   }
-  st->counter = 0;
 }
 
-// Block-sum NV doubles (fixed order) into dst[0 .. NV-1].  scratch: >= 32 * NV
-// doubles of shared memory.  Every thread of the block must call it.
-template <int NV>
-__device__ inline void block_sum(const double (&acc)[NV], double* dst, double* scratch) {
+// Sums of 8 values per thread over the block, in a fixed order, valid in lanes 0..7 of warp 0 (lane v:
+// value v).  A warp sums its 32 x 8 values in 9 additions per lane instead of 8 x 5: each of the first
+// three exchanges also halves the values a lane keeps.  (FP64 additions run at 2 lanes per SM and
+// clock, so the plain form cost each block of a pass about 2 us.)  scratch: kReduceScratch bytes of
+// shared memory.  Every thread of the block must call it.
+__device__ inline double block_sum8(const double (&acc)[8], double* scratch) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x + 31) >> 5;
+  double v[4];
+  {
+    const bool up = (lane & 16) != 0;
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    double s = warp_sum(acc[v]);
-    if (lane == 0) scratch[warp * NV + v] = s;
+    for (int i = 0; i < 4; ++i) {
+      const double keep = up ? acc[4 + i] : acc[i], send = up ? acc[i] : acc[4 + i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
   }
+  {
+    const bool up = (lane & 8) != 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const double keep = up ? v[2 + i] : v[i], send = up ? v[i] : v[2 + i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+  }
+  const bool up = (lane & 4) != 0;
+  const double keep = up ? v[1] : v[0], send = up ? v[0] : v[1];
+  double s = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  if ((lane & 3) == 0) scratch[warp * 8 + (lane >> 2)] = s;
   __syncthreads();
-  if (tid < NV) {
-    double s = 0;
-    for (int w = 0; w < nw; ++w) s += scratch[w * NV + tid];
-    dst[tid] = s;
+  double t = 0;
+  if (warp == 0) {
+    for (int w = lane >> 3; w < nw; w += 4) t += scratch[w * 8 + (lane & 7)];
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
   }
+  return t;
 }
 
 // After every block has written its partials: true in the one block that
@@ -186,25 +229,51 @@ __device__ inline bool last_block_arrived(DevStatus* st, unsigned int nblk) {
   return am_last;
 }
 
-// Block-sum NRED doubles (fixed order) and publish them as this block's
-// partials; the last block to arrive reduces all partials in index order and
-// evaluates the stopping test.  scratch: >= 32 * NRED doubles of shared memory.
+// Block-sum NRED doubles (fixed order) and publish them as this block's partials.  scratch:
+// kReduceScratch bytes of shared memory.
+__device__ inline void publish_partials(const double (&acc)[NRED], double* partials, double* scratch) {
+  const int bid = blockIdx.y * gridDim.x + blockIdx.x;
+  const double a8[8] = {acc[0], acc[1], acc[2], acc[3], acc[4], acc[5], acc[6], 0.0};
+  const double s = block_sum8(a8, scratch);
+  if (threadIdx.x < 8) partials[(size_t)bid * kPartStride + threadIdx.x] = s;
+}
+
+// Sum the partials of nblk blocks in a fixed order and evaluate the stopping
+// test, by one block: each thread takes every blockDim-th block's partials,
+// four 16-byte loads per block and four blocks in flight.
+__device__ inline void finalize_partials(int nblk, const double* partials, DevStatus* st, double* hist,
+                                         double* scratch) {
+  double a8[8];
+#pragma unroll
+  for (int v = 0; v < 8; ++v) a8[v] = 0;
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
+    const double2* q = reinterpret_cast<const double2*>(partials + (size_t)b * kPartStride);
+    double2 d[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) d[v] = __ldcg(q + v);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      a8[2 * v] += d[v].x;
+      if (v < 3) a8[2 * v + 1] += d[v].y;
+    }
+  }
+  const double t = block_sum8(a8, scratch);
+  // the sums of lanes 0..7 to one thread
+  double sums[NRED];
+#pragma unroll
+  for (int v = 0; v < NRED; ++v) sums[v] = __shfl_sync(0xffffffffu, t, v);
+  if (threadIdx.x == 0) finalize_eval(st, hist, sums);
+}
+
+// Publish this block's partials; the last block to arrive takes the sum and the
+// stopping test (passes that no kernel of the same evaluation follows).
 __device__ inline void reduce_and_finalize(const double (&acc)[NRED], double* partials, DevStatus* st,
                                            double* hist, double* scratch) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x + 31) >> 5;
   const int nblk = gridDim.x * gridDim.y;
-  const int bid = blockIdx.y * gridDim.x + blockIdx.x;
-  block_sum<NRED>(acc, partials + (size_t)bid * NRED, scratch);
+  publish_partials(acc, partials, scratch);
   if (!last_block_arrived(st, (unsigned)nblk)) return;
-  // deterministic: value v by warp (v mod nw), lanes stride over blocks
-  for (int v = warp; v < NRED; v += nw) {
-    double s = 0;
-    for (int b = lane; b < nblk; b += 32) s += __ldcg(partials + (size_t)b * NRED + v);
-    s = warp_sum(s);
-    if (lane == 0) scratch[v] = s;
-  }
-  __syncthreads();
-  if (tid == 0) finalize_eval(st, hist, scratch);
+  finalize_partials(nblk, partials, st, hist, scratch);
 }
 
 // ---- mbarriers and tensor (TMA) copies ------------------------------------------------------

@@ -2,165 +2,32 @@
 #pragma once
 #include <string.h>
 
-#include <map>
-#include <mutex>
-#include <type_traits>
-#include <utility>
-
-#include "launch.h"
+#include "launch_util.cuh"
 
 namespace hs {
 
-// Raise a kernel's dynamic shared-memory limit when a launch needs more than
-// it has been given so far on the current device (the attribute is per device,
-// so the record is keyed by device ordinal and kernel).  Launches recorded into
-// a graph capture therefore never call the attribute API: the first,
-// uncaptured, chunk of a solve has already set it.
-inline std::mutex& smem_mu() {
-  static std::mutex m;
-  return m;
-}
-inline std::map<std::pair<int, const void*>, size_t>& smem_set() {
-  static std::map<std::pair<int, const void*>, size_t> m;
-  return m;
-}
-template <typename K> static cudaError_t set_smem(K kernel, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const std::pair<int, const void*> key(dev, reinterpret_cast<const void*>(kernel));
-  std::lock_guard<std::mutex> lock(smem_mu());
-  size_t& have = smem_set()[key];
-  if (smem <= have) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) have = smem;
-  return e;
-}
-
-template <typename T, int TY, class MAT, int MODE, bool REAL, bool BATCH>
-static cudaError_t march_launch(const MarchArgs<T>& a, const MAT& m, dim3 g, int nthr, size_t smem,
-                                cudaStream_t s) {
-  auto k = k_march<T, TY, MAT, MODE, REAL, BATCH>;
+template <typename T, int TY, class MAT, int MODE>
+static cudaError_t march_one(const MarchArgs<T>& a, const MAT& m, dim3 g, int nthr, size_t smem, cudaStream_t s) {
+  auto k = k_march<T, TY, MAT, MODE>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   k<<<g, nthr, smem, s>>>(a, m);
   return cudaGetLastError();
 }
 
-// batched launches (zstride != 0) run the real-space force pass only
-template <typename T, int TY, class MAT, int MODE, bool REAL>
-static cudaError_t march_one(const MarchArgs<T>& a, const MAT& m, dim3 g, int nthr, size_t smem, cudaStream_t s) {
-  if constexpr (MODE == MODE_FORCE && REAL) {
-    if (a.zstride != 0) return march_launch<T, TY, MAT, MODE, REAL, true>(a, m, g, nthr, smem, s);
-  } else {
-    if (a.zstride != 0) return cudaErrorInvalidValue;
-  }
-  return march_launch<T, TY, MAT, MODE, REAL, false>(a, m, g, nthr, smem, s);
-}
-
-template <typename T, int TY, bool REAL>
+template <typename T, int TY>
 static cudaError_t march_ty(const MarchArgs<T>& a, bool iso, int mode, dim3 g, int nthr, size_t smem,
                             cudaStream_t s) {
-  if (mode == MODE_EMIT) {
-    if (REAL) return cudaErrorInvalidValue;
-    return march_one<T, TY, MatIso<T>, MODE_EMIT, false>(a, MatIso<T>{a.mat}, g, nthr, smem, s);
-  }
-  if (mode == MODE_FORCE_FIELDS) {  // last FP64 residual sweep of a refined solve
-    if constexpr (REAL && sizeof(T) == 8) {
-      if (iso) return march_one<T, TY, MatIso<T>, MODE_FORCE_FIELDS, REAL>(a, MatIso<T>{a.mat}, g, nthr, smem, s);
-      return march_one<T, TY, MatAniso<T>, MODE_FORCE_FIELDS, REAL>(a, MatAniso<T>{a.mat}, g, nthr, smem, s);
-    } else {
-      return cudaErrorInvalidValue;
-    }
-  }
-  if (iso) {
-    MatIso<T> m{a.mat};
-    if (mode == MODE_FORCE) return march_one<T, TY, MatIso<T>, MODE_FORCE, REAL>(a, m, g, nthr, smem, s);
-    return march_one<T, TY, MatIso<T>, MODE_FIELDS, REAL>(a, m, g, nthr, smem, s);
-  }
-  MatAniso<T> m{a.mat};
-  if (mode == MODE_FORCE) return march_one<T, TY, MatAniso<T>, MODE_FORCE, REAL>(a, m, g, nthr, smem, s);
-  return march_one<T, TY, MatAniso<T>, MODE_FIELDS, REAL>(a, m, g, nthr, smem, s);
-}
-
-// resident blocks per SM of the FP64 real-space force pass (single solves)
-template <int TY, class MAT>
-static cudaError_t march64_occ_one(int nthr, size_t smem, int* n) {
-  auto k = k_march<double, TY, MAT, MODE_FORCE, true, false>;
-  cudaError_t e = set_smem(k, smem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, nthr, smem);
-}
-template <int TY>
-static cudaError_t march64_occ_ty(bool iso, int nthr, size_t smem, int* n) {
-  return iso ? march64_occ_one<TY, MatIso<double>>(nthr, smem, n) : march64_occ_one<TY, MatAniso<double>>(nthr, smem, n);
-}
-
-template <typename T, bool REAL>
-static cudaError_t march_real(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 g, int nthr, size_t smem,
-                              cudaStream_t s) {
-  switch (ty) {
-    case 2: return march_ty<T, 2, REAL>(a, iso, mode, g, nthr, smem, s);
-    case 4: return march_ty<T, 4, REAL>(a, iso, mode, g, nthr, smem, s);
-    case 8: return march_ty<T, 8, REAL>(a, iso, mode, g, nthr, smem, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <int TY, class MATP, int MODE, int N1, bool BATCH>
-static cudaError_t stencil_launch(const MarchArgs<float>& a, const MATP& m, dim3 g, int nthr, size_t smem,
-                                  cudaStream_t s) {
-  auto k = k_stencil<TY, MATP, MODE, N1, BATCH>;
-  cudaError_t e = set_smem(k, smem);
-  if (e != cudaSuccess) return e;
-  k<<<g, nthr, smem, s>>>(a, m);
-  return cudaGetLastError();
-}
-
-// batched launches (zstride != 0) run the force pass only
-template <int TY, class MATP, int MODE, int N1 = 0>
-static cudaError_t stencil_one(const MarchArgs<float>& a, const MATP& m, dim3 g, int nthr, size_t smem,
-                               cudaStream_t s) {
-  if constexpr (MODE == MODE_FORCE) {
-    if (a.zstride != 0) return stencil_launch<TY, MATP, MODE, N1, true>(a, m, g, nthr, smem, s);
-  } else {
-    if (a.zstride != 0) return cudaErrorInvalidValue;
-  }
-  return stencil_launch<TY, MATP, MODE, N1, false>(a, m, g, nthr, smem, s);
-}
-
-template <int TY>
-static cudaError_t stencil_ty(const MarchArgs<float>& a, bool iso, int mode, dim3 g, int nthr, size_t smem,
-                              cudaStream_t s) {
-  if (iso) {
-    MatIsoP m{a.mat};
-    if constexpr (TY == 4) {
-      if (mode == MODE_FORCE && a.n1 == 256 && nthr == 256)
-        return stencil_one<TY, MatIsoP, MODE_FORCE, 256>(a, m, g, nthr, smem, s);
-    }
-    if (mode == MODE_FORCE) return stencil_one<TY, MatIsoP, MODE_FORCE>(a, m, g, nthr, smem, s);
-    return stencil_one<TY, MatIsoP, MODE_FIELDS>(a, m, g, nthr, smem, s);
-  }
-  MatAnisoP m{a.mat};
-  if constexpr (TY == 4) {
-    if (mode == MODE_FORCE && a.n1 == 256 && nthr == 256)
-      return stencil_one<TY, MatAnisoP, MODE_FORCE, 256>(a, m, g, nthr, smem, s);
-  }
-  if (mode == MODE_FORCE) return stencil_one<TY, MatAnisoP, MODE_FORCE>(a, m, g, nthr, smem, s);
-  return stencil_one<TY, MatAnisoP, MODE_FIELDS>(a, m, g, nthr, smem, s);
-}
-
-// FP32 real-space pass (FORCE / FIELDS on a real displacement field); a
-// template so that only the unit that launches it instantiates its kernels
-template <int UNUSED = 0>
-static cudaError_t stencil_f32(const MarchArgs<float>& a, bool iso, int ty, int mode, dim3 g, int nthr,
-                               size_t smem, cudaStream_t s) {
-  if (mode != MODE_FORCE && mode != MODE_FIELDS) return cudaErrorInvalidValue;
-  switch (ty) {
-    case 2: return stencil_ty<2>(a, iso, mode, g, nthr, smem, s);
-    case 4: return stencil_ty<4>(a, iso, mode, g, nthr, smem, s);
-    case 8: return stencil_ty<8>(a, iso, mode, g, nthr, smem, s);
+  const MatIso<T> mi{a.mat};
+  const MatAniso<T> ma{a.mat};
+  switch (mode) {
+    case MODE_EMIT: return march_one<T, TY, MatIso<T>, MODE_EMIT>(a, mi, g, nthr, smem, s);
+    case MODE_FORCE:
+      return iso ? march_one<T, TY, MatIso<T>, MODE_FORCE>(a, mi, g, nthr, smem, s)
+                 : march_one<T, TY, MatAniso<T>, MODE_FORCE>(a, ma, g, nthr, smem, s);
+    case MODE_FIELDS:
+      return iso ? march_one<T, TY, MatIso<T>, MODE_FIELDS>(a, mi, g, nthr, smem, s)
+                 : march_one<T, TY, MatAniso<T>, MODE_FIELDS>(a, ma, g, nthr, smem, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -175,14 +42,6 @@ static cudaError_t col_one(const ColArgs<T>& a, dim3 g, int nthr, size_t smem, c
   if (e != cudaSuccess) return e;
   k<<<g, nthr, smem, s>>>(a);
   return cudaGetLastError();
-}
-
-// real-displacement passes: the packed FP32 kernel, or k_march for FP64
-template <typename T>
-static cudaError_t march_real_dispatch(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 g, int nthr,
-                                      size_t smem, cudaStream_t s) {
-  if constexpr (std::is_same<T, float>::value) return stencil_f32<>(a, iso, ty, mode, g, nthr, smem, s);
-  else return march_real<double, true>(a, iso, ty, mode, g, nthr, smem, s);
 }
 
 template <typename T, int CT, int LF = 0, int NT = 0>
@@ -328,18 +187,20 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
 #define HS_INSTANTIATE(T, REALOK, CT, NT)                                                                 \
   namespace hs {                                                                                         \
   template <>                                                                                            \
-  cudaError_t launch_march<T>(const MarchArgs<T>& a, bool iso, int ty, int mode, bool real, dim3 grid,  \
-                              int nthr, size_t smem, cudaStream_t s) {                                   \
-    if (a.ids == nullptr || a.mat == nullptr || a.st == nullptr || a.partials == nullptr)                \
+  cudaError_t launch_march<T>(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 grid, int nthr, size_t smem, \
+                              cudaStream_t s) {                                                          \
+    if (a.ids == nullptr || a.mat == nullptr || a.st == nullptr || a.partials == nullptr || a.in == nullptr || \
+        a.zstride != 0)                                                                                  \
       return cudaErrorInvalidValue;                                                                      \
-    if (real && a.ureal == nullptr) return cudaErrorInvalidValue;                                        \
-    if (!real && a.in == nullptr) return cudaErrorInvalidValue;                                          \
     if (mode == MODE_EMIT && a.u64 == nullptr) return cudaErrorInvalidValue;                             \
-    if (mode == MODE_FORCE && !real && a.out == nullptr) return cudaErrorInvalidValue;                   \
-    if ((mode == MODE_FIELDS || mode == MODE_FORCE_FIELDS) && (a.eps_out == nullptr || a.sig_out == nullptr)) \
-      return cudaErrorInvalidValue;                                                                      \
-    if (real) return march_real_dispatch(a, iso, ty, mode, grid, nthr, smem, s);                         \
-    return march_real<T, false>(a, iso, ty, mode, grid, nthr, smem, s);                                  \
+    if (mode == MODE_FORCE && a.out == nullptr) return cudaErrorInvalidValue;                            \
+    if (mode == MODE_FIELDS && (a.eps_out == nullptr || a.sig_out == nullptr)) return cudaErrorInvalidValue; \
+    switch (ty) {                                                                                        \
+      case 2: return march_ty<T, 2>(a, iso, mode, grid, nthr, smem, s);                                  \
+      case 4: return march_ty<T, 4>(a, iso, mode, grid, nthr, smem, s);                                  \
+      case 8: return march_ty<T, 8>(a, iso, mode, grid, nthr, smem, s);                                  \
+      default: return cudaErrorInvalidValue;                                                             \
+    }                                                                                                    \
   }                                                                                                      \
   template <>                                                                                            \
   cudaError_t launch_col<T>(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem,      \
@@ -358,16 +219,6 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
       return cudaErrorInvalidValue;                                                                      \
     if (ct != (CT) / 2 || plan_ext(a.plan) || a.state_smem) return cudaErrorNotSupported;               \
     return colp_dispatch<T, (CT) / 2, NT>(a, mode, col_length(a, mode), grid, nthr, smem, s, nullptr);   \
-  }                                                                                                      \
-  template <>                                                                                            \
-  cudaError_t march_blocks_per_sm<T>(bool iso, int ty, int nthr, size_t smem, int* n) {                 \
-    if (sizeof(T) != 8) return cudaErrorNotSupported;                                                    \
-    switch (ty) {                                                                                        \
-      case 2: return march64_occ_ty<2>(iso, nthr, smem, n);                                              \
-      case 4: return march64_occ_ty<4>(iso, nthr, smem, n);                                              \
-      case 8: return march64_occ_ty<8>(iso, nthr, smem, n);                                              \
-      default: return cudaErrorInvalidValue;                                                             \
-    }                                                                                                    \
   }                                                                                                      \
   template <>                                                                                            \
   cudaError_t colp_blocks_per_sm<T>(int mode, int L, int ct, int nthr, size_t smem, int* n) {            \

@@ -6,15 +6,56 @@
 #include "colpass.cuh"
 #include "march.cuh"
 #include "rowpass.cuh"
-#include "stencil.cuh"
 
 namespace hs {
 
-// mode: MODE_FORCE / MODE_FIELDS / MODE_EMIT; real: input is the FP64 real
-// displacement field (only for T = double).
+// Entries of the phase tables (layouts in common.cuh): an isotropic phase, or the 21 upper-triangle entries
+// of a 6x6 matrix, row-major; rounded to T, then scaled (exactly).
+inline void pack_iso(double lam, double mu, double* out) {
+  out[0] = lam * kTabScale<double>;
+  out[1] = mu * kTabScale<double>;
+}
+inline void pack_iso(double lam, double mu, float* out) {
+  out[0] = out[1] = (float)lam * kTabScale<float>;
+  out[2] = out[3] = (float)mu * kTabScale<float>;
+}
+template <typename T> void pack_upper(const double* C, T* out) {
+  for (int i = 0; i < 6; ++i)
+    for (int j = i; j < 6; ++j) *out++ = (T)C[i * 6 + j] * kTabScale<T>;
+}
+
+// fused x pass (xfuse = 1); mode: MODE_FORCE / MODE_FIELDS / MODE_EMIT
 template <typename T>
-cudaError_t launch_march(const MarchArgs<T>& a, bool iso, int ty, int mode, bool real, dim3 grid, int nthr,
-                         size_t smem, cudaStream_t s);
+cudaError_t launch_march(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 grid, int nthr, size_t smem,
+                         cudaStream_t s);
+
+// Compile-time row pitch of the pass on a real displacement: the FP32 force pass with tiles of 4 rows and
+// rows that bulk copies take (N1 a multiple of 8) runs the next of four; 0: none.
+inline int real_pitch_class(bool f64, int ty, int mode, int n1) {
+  if (f64 || ty != 4 || mode != MODE_FORCE || n1 % 8 != 0) return 0;
+  return n1 <= 64 ? 64 : n1 <= 128 ? 128 : n1 <= 256 ? 256 : 512;
+}
+// Its row pitch in shared memory.
+inline int real_pitch(bool f64, int ty, int mode, int n1) {
+  const int c = real_pitch_class(f64, ty, mode, n1);
+  return c > 0 ? c : (n1 + 7) & ~7;
+}
+
+// The pass on a real displacement field (k_real): mode MODE_FORCE / MODE_FIELDS / MODE_FORCE_FIELDS (FP64
+// only); a.xp as real_pitch() gives it.  occ: not null: the resident blocks per SM instead of a launch.
+template <typename T, bool ISO>
+cudaError_t launch_real_law(const MarchArgs<T>& a, int ty, int mode, dim3 grid, int nthr, size_t smem, cudaStream_t s,
+                            int* occ);
+template <> cudaError_t launch_real_law<float, true>(const MarchArgs<float>&, int, int, dim3, int, size_t, cudaStream_t, int*);
+template <> cudaError_t launch_real_law<float, false>(const MarchArgs<float>&, int, int, dim3, int, size_t, cudaStream_t, int*);
+template <> cudaError_t launch_real_law<double, true>(const MarchArgs<double>&, int, int, dim3, int, size_t, cudaStream_t, int*);
+template <> cudaError_t launch_real_law<double, false>(const MarchArgs<double>&, int, int, dim3, int, size_t, cudaStream_t, int*);
+template <typename T>
+cudaError_t launch_real(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 grid, int nthr, size_t smem,
+                        cudaStream_t s, int* occ = nullptr) {
+  return iso ? launch_real_law<T, true>(a, ty, mode, grid, nthr, smem, s, occ)
+             : launch_real_law<T, false>(a, ty, mode, grid, nthr, smem, s, occ);
+}
 
 template <typename T>
 cudaError_t launch_col(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s);
@@ -26,10 +67,6 @@ template <typename T>
 cudaError_t launch_colp(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s);
 template <typename T>
 cudaError_t colp_blocks_per_sm(int mode, int L, int ct, int nthr, size_t smem, int* n);
-
-// resident blocks per SM of the FP64 real-space force pass of a single solve (T = double only)
-template <typename T>
-cudaError_t march_blocks_per_sm(bool iso, int ty, int nthr, size_t smem, int* n);
 
 // mode: ROW_C2R / ROW_R2C; grid.x persistent blocks per item, grid.z items (batched launches)
 template <typename T>

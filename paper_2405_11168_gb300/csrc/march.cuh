@@ -1,11 +1,11 @@
-// Real-space pass of the tetrahedral-stencil basic scheme, marching along z.
+// Fused x pass (xfuse = 1) of the tetrahedral-stencil basic scheme, marching along z; the pass on a
+// real displacement field (the default and the FP64 sweeps) is in real.cuh.
 //
 // One block owns a tile of TY corner rows (y) of one z-chunk and all N1 x
 // positions (thread x <-> column x).  For every voxel plane p it
-//   1. brings the corner plane p (rows y0-1 .. y0+TY) into shared memory:
-//      either by an inverse real FFT along x of the y/z-transformed state
-//      (two real rows packed in one complex sequence), or (REAL = true) by
-//      plain loads of a real FP64 displacement field;
+//   1. brings the corner plane p (rows y0-1 .. y0+TY) into shared memory by an
+//      inverse real FFT along x of the y/z-transformed state (two real rows
+//      packed in one complex sequence);
 //   2. computes, per voxel, the T1 and T2 strains of the two inscribed
 //      tetrahedra (Eqs. deps, DA1-DA2; T1 = corners whose offset signs
 //      multiply to +1, T2 = the centrally symmetric set), the stresses
@@ -16,7 +16,7 @@
 //      for corner planes p-1 and p; contributions to column x-1 go left by
 //      warp shuffle (lane 0's through shared memory);
 //   4. when corner plane p-1 is complete: forward real FFT along x (packed
-//      pairs) and store (FORCE), or store the real force (REAL FORCE).
+//      pairs) and store (FORCE).
 // FIELDS writes eps = E + 1/2(deps^T1 + deps^T2) and sigma = 1/2(sigma^T1 +
 // sigma^T2) (Eq. final_fields) instead; EMIT adds the inverse-transformed
 // displacement into an FP64 real field.
@@ -28,7 +28,7 @@
 
 namespace hs {
 
-// MODE_FORCE_FIELDS: MODE_FORCE that also writes the fields of MODE_FIELDS (the
+// MODE_FORCE_FIELDS (k_real only): MODE_FORCE that also writes the fields of MODE_FIELDS (the
 // last FP64 residual sweep of a refined solve)
 enum { MODE_FORCE = 0, MODE_FIELDS = 1, MODE_EMIT = 2, MODE_FORCE_FIELDS = 3 };
 
@@ -50,9 +50,12 @@ template <typename T> struct MarchArgs {
   void* sig_out;
   int out_f32;
   double* u64;           // EMIT: += u
-  const T* ureal;        // REAL: input displacement [3][n3][n2][n1]
-  void* fout;            // REAL FORCE: real force [3][n3][n2][n1], float if fout_f32 else T
+  const T* ureal;        // k_real: input displacement [3][n3][n2][n1]
+  void* fout;            // k_real, FORCE: real force [3][n3][n2][n1], float if fout_f32 else T
   int fout_f32;
+  int xp;                // k_real: row pitch in shared memory (a multiple of 8, >= n1)
+  int defer;             // k_real: 1 = the forward row pass that follows sums the partials and takes the stopping test
+  int bulk;              // k_real: 1 = planes arrive by bulk copies (n1 a multiple of 8, inputs 16-byte aligned)
   int skip_if_done;
   const double* Edev;    // not null: the macroscopic strain is read here (applied-stress control)
   const T* sig0;         // not null: lambda(ph) : eps0(ph) per phase, Voigt [nphase][6] (eigenstrain)
@@ -181,14 +184,14 @@ __device__ __forceinline__ void tetra_strain_fast(const T (&u)[2][2][2][3], cons
 
 // Shared-memory layout of k_march (host and device use the same function).
 struct MarchLayout {
-  size_t ring, fbuf, stage, ids, src, edge, red, bar, total;
+  size_t ring, fbuf, stage, ids, src, edge, red, total;
   int n1i, n1s;  // row pitches (elements) of the ids and source stages
 };
 
 __host__ __device__ inline size_t hs_align16(size_t x) { return (x + 15) & ~size_t(15); }
 
-__host__ __device__ inline MarchLayout march_layout(int n1, int P, int nthr, int ty, int mode, bool real,
-                                                    bool has_src, int tsize) {
+__host__ __device__ inline MarchLayout march_layout(int n1, int P, int nthr, int ty, int mode, bool has_src,
+                                                    int tsize) {
   MarchLayout L;
   const int NR = ty + 2, NSI = 3 * NR / 2, NSF = 3 * ty / 2;
   const size_t cs = 2 * (size_t)tsize;
@@ -196,11 +199,11 @@ __host__ __device__ inline MarchLayout march_layout(int n1, int P, int nthr, int
   L.n1s = (n1 + 3) & ~3;
   size_t off = 0;
   L.ring = off;
-  off += hs_align16(real ? (size_t)tsize * 3 * 3 * NR * n1 : cs * 2 * NSI * rpitch(n1));
+  off += hs_align16(cs * 2 * NSI * rpitch(n1));
   L.fbuf = off;
-  off += hs_align16((real || mode != MODE_FORCE) ? 0 : cs * NSF * rpitch(n1));
+  off += hs_align16(mode != MODE_FORCE ? 0 : cs * NSF * rpitch(n1));
   L.stage = off;
-  off += hs_align16(real ? 0 : cs * 3 * NR * (size_t)P);
+  off += hs_align16(cs * 3 * NR * (size_t)P);
   L.ids = off;
   off += hs_align16(mode == MODE_EMIT ? 0 : (size_t)2 * 2 * (ty + 1) * L.n1i);
   L.src = off;
@@ -208,32 +211,27 @@ __host__ __device__ inline MarchLayout march_layout(int n1, int P, int nthr, int
   L.edge = off;
   off += hs_align16((size_t)tsize * (nthr / 32) * (ty + 1) * 12);
   L.red = off;
-  off += 32 * NRED * 8;
-  L.bar = off;  // three mbarriers (bulk plane copies of the FP32 real-space pass)
-  off += 32;
+  off += kReduceScratch;
   L.total = off;
   return L;
 }
 
 template <typename T> struct MarchPtrs {
   const typename cplx_t<T>::type* in;
-  const T* ureal;
   const uint16_t* ids;
   const float* src;
   typename cplx_t<T>::type* stage;
-  T* rring;
   uint16_t* sids;
   float* ssrc;
   int n1, n2, n3, P, y0, n1i, n1s;
 };
 
 // Asynchronous prefetch of one plane's inputs: u rows of corner plane pu
-// (complex: into the staging rows; REAL: into ring slot rslot), ids rows of
-// voxel plane pu into ids buffer ib, source rows of output plane ps into
+// into the staging rows, ids rows of voxel plane pu into ids buffer ib, source rows of output plane ps into
 // source buffer ib (ps < 0: none).  Ends with a commit of the copy group.
-template <typename T, int TY, bool REAL>
-__device__ __forceinline__ void march_prefetch(const MarchPtrs<T>& m, int tid, int nthr, int pu, int rslot, int ib,
-                                               int ps, bool want_ids) {
+template <typename T, int TY>
+__device__ __forceinline__ void march_prefetch(const MarchPtrs<T>& m, int tid, int nthr, int pu, int ib, int ps,
+                                               bool want_ids) {
   using C = typename cplx_t<T>::type;
   constexpr int NR = TY + 2;
   constexpr int EPC = 16 / (int)sizeof(C);
@@ -241,35 +239,14 @@ __device__ __forceinline__ void march_prefetch(const MarchPtrs<T>& m, int tid, i
   const size_t rplane = (size_t)n2 * n1, rcomp = (size_t)n3 * rplane;
   const size_t plane_stride = (size_t)n2 * P, comp_stride = (size_t)n3 * plane_stride;
   const int gz = ((pu % n3) + n3) % n3;
-  if (REAL) {
-    constexpr int EPR = 16 / (int)sizeof(T);  // real values per 16-byte chunk
-    T* dst0 = m.rring + (size_t)rslot * 3 * NR * n1;
-    if (n1 % EPR == 0) {
-      const int nch = n1 / EPR;
-      for (int i = tid; i < 3 * NR * nch; i += nthr) {
-        const int r = i / nch, ch = i - r * nch;
-        const int c = r / NR, j = r - c * NR;
-        const int gy = (y0 - 1 + j + n2) % n2;
-        cp_async16(dst0 + (size_t)r * n1 + EPR * ch,
-                   m.ureal + c * rcomp + (size_t)gz * rplane + (size_t)gy * n1 + EPR * ch);
-      }
-    } else if (tid < n1) {
-      for (int r = 0; r < 3 * NR; ++r) {
-        const int c = r / NR, j = r - c * NR;
-        const int gy = (y0 - 1 + j + n2) % n2;
-        dst0[(size_t)r * n1 + tid] = m.ureal[c * rcomp + (size_t)gz * rplane + (size_t)gy * n1 + tid];
-      }
-    }
-  } else {
-    const int nh = n1 / 2 + 1;
-    const int nch = (nh + EPC - 1) / EPC;
-    for (int i = tid; i < 3 * NR * nch; i += nthr) {
-      const int r = i / nch, ch = i - r * nch;
-      const int c = r / NR, j = r - c * NR;
-      const int gy = (y0 - 1 + j + n2) % n2;
-      cp_async16(m.stage + (size_t)r * P + ch * EPC,
-                 m.in + c * comp_stride + (size_t)gz * plane_stride + (size_t)gy * P + ch * EPC);
-    }
+  const int nh = n1 / 2 + 1;
+  const int nch = (nh + EPC - 1) / EPC;
+  for (int i = tid; i < 3 * NR * nch; i += nthr) {
+    const int r = i / nch, ch = i - r * nch;
+    const int c = r / NR, j = r - c * NR;
+    const int gy = (y0 - 1 + j + n2) % n2;
+    cp_async16(m.stage + (size_t)r * P + ch * EPC,
+               m.in + c * comp_stride + (size_t)gz * plane_stride + (size_t)gy * P + ch * EPC);
   }
   if (want_ids) {
     uint16_t* d = m.sids + (size_t)ib * (TY + 1) * m.n1i;
@@ -333,32 +310,22 @@ __device__ __forceinline__ void march_pack(const MarchPtrs<T>& m, typename cplx_
   __syncthreads();
 }
 
-template <typename T, int TY, bool REAL>
-__device__ __forceinline__ T march_u(const typename cplx_t<T>::type* ring, const T* rring, int n1, int slot, int c,
-                                     int j, int xx) {
+template <typename T, int TY>
+__device__ __forceinline__ T march_u(const typename cplx_t<T>::type* ring, int n1, int slot, int c, int j, int xx) {
   constexpr int NR = TY + 2;
   constexpr int NSI = 3 * NR / 2;
-  if (REAL) return rring[((size_t)slot * 3 * NR + c * NR + j) * n1 + xx];
   const int r = c * NR + j;
   const auto z = ring[(slot * NSI + (r >> 1)) * rpitch(n1) + rpad(xx)];
   return (r & 1) ? z.y : z.x;
 }
 
-// BATCH: a batched launch (grid.z items, every workspace pointer moved per item); a single
-// solve's launch uses the arguments as they come.
-// Blocks of up to 512 threads; the FP64 tile of 8 rows takes blocks of at most 256 (N1 <= 256), so
-// that its registers (up to 255) hold the FP64 sweep without spills.
-template <typename T, int TY, class MAT, int MODE, bool REAL, bool BATCH = false>
-__global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_march(const MarchArgs<T> a_,
-                                                                                    const MAT mat_) {
+template <typename T, int TY, class MAT, int MODE>
+__global__ void __launch_bounds__(512) k_march(const MarchArgs<T> a, const MAT mat) {
   using C = typename cplx_t<T>::type;
   constexpr int NR = TY + 2;          // corner rows per plane (1 halo row each side)
   constexpr int NSI = 3 * NR / 2;     // packed complex sequences per plane
   constexpr int NSF = 3 * TY / 2;     // packed sequences of the output force
   constexpr int EPC = 16 / (int)sizeof(C);
-  const MarchArgs<T> a = BATCH ? march_item_args(a_) : a_;
-  MAT mat = mat_;
-  if (BATCH) mat.tab = a.mat;
   if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int n1 = a.n1, n2 = a.n2, n3 = a.n3, P = a.P, nh = n1 / 2 + 1;
@@ -377,9 +344,8 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
   const FftPlan plan = a.plan1;
   const bool has_src = (a.src != nullptr);
 
-  const MarchLayout lay = march_layout(n1, P, nthr, TY, MODE, REAL, has_src, (int)sizeof(T));
+  const MarchLayout lay = march_layout(n1, P, nthr, TY, MODE, has_src, (int)sizeof(T));
   C* ring = reinterpret_cast<C*>(smraw + lay.ring);      // complex: [2][NSI][n1]
-  T* rring = reinterpret_cast<T*>(smraw + lay.ring);     // REAL: [3][3*NR][n1]
   C* fbuf = reinterpret_cast<C*>(smraw + lay.fbuf);      // [NSF][n1]
   C* stage = reinterpret_cast<C*>(smraw + lay.stage);    // [3*NR][P] raw rows of the next plane
   uint16_t* sids = reinterpret_cast<uint16_t*>(smraw + lay.ids);  // [2][TY+1][n1i]
@@ -394,11 +360,9 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
 
   MarchPtrs<T> mp;
   mp.in = in;
-  mp.ureal = a.ureal;
   mp.ids = ids;
   mp.src = a.src;
   mp.stage = stage;
-  mp.rring = rring;
   mp.sids = sids;
   mp.ssrc = ssrc;
   mp.n1 = n1;
@@ -411,12 +375,12 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
 
   if (MODE == MODE_EMIT) {
     double* __restrict__ u64 = a.u64;
-    march_prefetch<T, TY, REAL>(mp, tid, nthr, z0, 0, 0, -1, false);
+    march_prefetch<T, TY>(mp, tid, nthr, z0, 0, -1, false);
     for (int p = z0; p < z0 + zc; ++p) {
       cp_async_wait_all();
       __syncthreads();
       march_pack<T, TY>(mp, ring, x, xact, 0);
-      if (p + 1 < z0 + zc) march_prefetch<T, TY, REAL>(mp, tid, nthr, p + 1, 0, 0, -1, false);
+      if (p + 1 < z0 + zc) march_prefetch<T, TY>(mp, tid, nthr, p + 1, 0, -1, false);
       HS_FFT_ROWS(true, ring, rpitch(n1), NSI, plan, tw1, tid, nthr);
       __syncthreads();
       if (xact) {
@@ -424,7 +388,7 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
         for (int c = 0; c < 3; ++c)
 #pragma unroll
           for (int r = 0; r < TY; ++r)
-            u64[c * rcomp + (size_t)p * rplane + (size_t)(y0 + r) * n1 + x] += (double)march_u<T, TY, REAL>(ring, rring, n1, 0, c, r + 1, x);
+            u64[c * rcomp + (size_t)p * rplane + (size_t)(y0 + r) * n1 + x] += (double)march_u<T, TY>(ring, n1, 0, c, r + 1, x);
       }
       __syncthreads();
     }
@@ -450,37 +414,23 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
   const int src_warp = ((x + 1) % n1) >> 5;
 
   // prologue: plane z0-1, then the prefetch of plane z0
-  if (REAL) {
-    march_prefetch<T, TY, REAL>(mp, tid, nthr, z0 - 1, 0, 0, -1, false);
-    march_prefetch<T, TY, REAL>(mp, tid, nthr, z0, 1, 0, -1, true);
-  } else {
-    march_prefetch<T, TY, REAL>(mp, tid, nthr, z0 - 1, 0, 0, -1, false);
-    cp_async_wait_all();
-    __syncthreads();
-    march_pack<T, TY>(mp, ring, x, xact, 0);
-    march_prefetch<T, TY, REAL>(mp, tid, nthr, z0, 0, 0, -1, true);
-    HS_FFT_ROWS(true, ring, rpitch(n1), NSI, plan, tw1, tid, nthr);
-    __syncthreads();
-  }
-  constexpr bool FORCE_LIKE = (MODE == MODE_FORCE || MODE == MODE_FORCE_FIELDS);
-  const int pend = FORCE_LIKE ? z0 + zc : z0 + zc - 1;
+  march_prefetch<T, TY>(mp, tid, nthr, z0 - 1, 0, -1, false);
+  cp_async_wait_all();
+  __syncthreads();
+  march_pack<T, TY>(mp, ring, x, xact, 0);
+  march_prefetch<T, TY>(mp, tid, nthr, z0, 0, -1, true);
+  HS_FFT_ROWS(true, ring, rpitch(n1), NSI, plan, tw1, tid, nthr);
+  __syncthreads();
+  const int pend = MODE == MODE_FORCE ? z0 + zc : z0 + zc - 1;
   for (int p = z0; p <= pend; ++p) {
     const int ib = (p - z0) & 1;  // ids buffer of voxel plane p, source buffer of output plane p-1
-    int sc, sp;
     cp_async_wait_all();
     __syncthreads();
-    if (REAL) {
-      sc = (p - z0 + 1) % 3;
-      sp = (p - z0) % 3;
-      if (p < pend) march_prefetch<T, TY, REAL>(mp, tid, nthr, p + 1, (p - z0 + 2) % 3, ib ^ 1, FORCE_LIKE ? p : -1, true);
-    } else {
-      sc = (p - z0 + 1) & 1;
-      sp = sc ^ 1;
-      march_pack<T, TY>(mp, ring, x, xact, sc);
-      if (p < pend) march_prefetch<T, TY, REAL>(mp, tid, nthr, p + 1, 0, ib ^ 1, FORCE_LIKE ? p : -1, true);
-      HS_FFT_ROWS(true, ring + sc * NSI * rpitch(n1), rpitch(n1), NSI, plan, tw1, tid, nthr);
-      __syncthreads();
-    }
+    const int sc = (p - z0 + 1) & 1, sp = sc ^ 1;
+    march_pack<T, TY>(mp, ring, x, xact, sc);
+    if (p < pend) march_prefetch<T, TY>(mp, tid, nthr, p + 1, ib ^ 1, MODE == MODE_FORCE ? p : -1, true);
+    HS_FFT_ROWS(true, ring + sc * NSI * rpitch(n1), rpitch(n1), NSI, plan, tw1, tid, nthr);
+    __syncthreads();
     const int pz = p % n3;
     const bool own_plane = p < z0 + zc;
     const uint16_t* idrow = sids + (size_t)ib * (TY + 1) * lay.n1i;
@@ -489,10 +439,10 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
     T uc[2][3][2];  // cached corner values of row jj: [ox][comp][oz]
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      uc[0][c][0] = march_u<T, TY, REAL>(ring, rring, n1, sc, c, 0, xr);
-      uc[0][c][1] = march_u<T, TY, REAL>(ring, rring, n1, sp, c, 0, xr);
-      uc[1][c][0] = march_u<T, TY, REAL>(ring, rring, n1, sc, c, 0, xmr);
-      uc[1][c][1] = march_u<T, TY, REAL>(ring, rring, n1, sp, c, 0, xmr);
+      uc[0][c][0] = march_u<T, TY>(ring, n1, sc, c, 0, xr);
+      uc[0][c][1] = march_u<T, TY>(ring, n1, sp, c, 0, xr);
+      uc[1][c][0] = march_u<T, TY>(ring, n1, sc, c, 0, xmr);
+      uc[1][c][1] = march_u<T, TY>(ring, n1, sp, c, 0, xmr);
     }
 #pragma unroll
     for (int jj = 1; jj <= TY + 1; ++jj) {
@@ -505,10 +455,10 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
           u[ox][1][0][c] = uc[ox][c][0];
           u[ox][1][1][c] = uc[ox][c][1];
         }
-        const T v00 = march_u<T, TY, REAL>(ring, rring, n1, sc, c, jj, xr);
-        const T v01 = march_u<T, TY, REAL>(ring, rring, n1, sp, c, jj, xr);
-        const T v10 = march_u<T, TY, REAL>(ring, rring, n1, sc, c, jj, xmr);
-        const T v11 = march_u<T, TY, REAL>(ring, rring, n1, sp, c, jj, xmr);
+        const T v00 = march_u<T, TY>(ring, n1, sc, c, jj, xr);
+        const T v01 = march_u<T, TY>(ring, n1, sp, c, jj, xr);
+        const T v10 = march_u<T, TY>(ring, n1, sc, c, jj, xmr);
+        const T v11 = march_u<T, TY>(ring, n1, sp, c, jj, xmr);
         u[0][0][0][c] = v00; u[0][0][1][c] = v01; u[1][0][0][c] = v10; u[1][0][1][c] = v11;
         uc[0][c][0] = v00; uc[0][c][1] = v01; uc[1][c][0] = v10; uc[1][c][1] = v11;
       }
@@ -564,29 +514,6 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
         if (acc_sig) {
 #pragma unroll
           for (int i = 0; i < 6; ++i) sacc[i] += sv[i];
-        }
-        if constexpr (MODE == MODE_FORCE_FIELDS) {
-          // eps = 1/2 (eps^T1 + eps^T2) (tensor components), sigma = 1/2 (sigma^T1 + sigma^T2):
-          // T1's halves are stored, T2's added to them
-          if (acc_sig) {
-            const size_t o = (size_t)pz * rplane + (size_t)((y0 + jj - 1) % n2) * n1 + x;
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-              const T eh = T(0.5) * ev[i] * (i < 3 ? T(1) : T(0.5));
-              const T sh = T(0.5) * sv[i];
-              if (a.out_f32) {
-                float* ep = reinterpret_cast<float*>(a.eps_out) + i * rcomp + o;
-                float* sp = reinterpret_cast<float*>(a.sig_out) + i * rcomp + o;
-                if (tt == 0) { *ep = (float)eh; *sp = (float)sh; }
-                else { *ep = (float)((T)*ep + eh); *sp = (float)((T)*sp + sh); }
-              } else {
-                double* ep = reinterpret_cast<double*>(a.eps_out) + i * rcomp + o;
-                double* sp = reinterpret_cast<double*>(a.sig_out) + i * rcomp + o;
-                if (tt == 0) { *ep = (double)eh; *sp = (double)sh; }
-                else { *ep += (double)eh; *sp += (double)sh; }
-              }
-            }
-          }
         }
         T l0[3], l1[3];
         // per force component k: (sigma_1k, sigma_2k, sigma_3k)
@@ -667,49 +594,36 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
 #pragma unroll
           for (int r = 0; r < TY; ++r) facc += Fp[r][c] * Fp[r][c];
       }
-      if (REAL) {
-        if (xact && a.fout != nullptr) {
+      if (xact) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int r = 0; r < TY; ++r) {
-              const size_t o = c * rcomp + (size_t)zp * rplane + (size_t)(y0 + r) * n1 + x;
-              if (a.fout_f32) reinterpret_cast<float*>(a.fout)[o] = (float)Fp[r][c];
-              else reinterpret_cast<T*>(a.fout)[o] = Fp[r][c];
-            }
-        }
-      } else {
-        if (xact) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int r = 0; r < TY; r += 2) {
-              C z;
-              z.x = Fp[r][c];
-              z.y = Fp[r + 1][c];
-              fbuf[((c * TY + r) >> 1) * rpitch(n1) + rpad(x)] = z;
-            }
-        }
-        __syncthreads();
-        HS_FFT_ROWS(false, fbuf, rpitch(n1), NSF, plan, tw1, tid, nthr);
-        __syncthreads();
-        if (x < nh) {
-          const int k = x;
-#pragma unroll
-          for (int q = 0; q < NSF; ++q) {
-            const C Zk = fbuf[q * rpitch(n1) + rpad(k)];
-            const C Zn = fbuf[q * rpitch(n1) + rpad(k == 0 ? 0 : n1 - k)];
-            C A, B;
-            A.x = T(0.5) * (Zk.x + Zn.x);
-            A.y = T(0.5) * (Zk.y - Zn.y);
-            B.x = T(0.5) * (Zk.y + Zn.y);
-            B.y = T(0.5) * (Zn.x - Zk.x);
-            const int ra = 2 * q;
-            const int c = ra / TY, r = ra - c * TY;
-            const size_t o = c * comp_stride + (size_t)zp * plane_stride + (size_t)(y0 + r) * P + k;
-            out[o] = A;
-            out[o + P] = B;
+          for (int r = 0; r < TY; r += 2) {
+            C z;
+            z.x = Fp[r][c];
+            z.y = Fp[r + 1][c];
+            fbuf[((c * TY + r) >> 1) * rpitch(n1) + rpad(x)] = z;
           }
+      }
+      __syncthreads();
+      HS_FFT_ROWS(false, fbuf, rpitch(n1), NSF, plan, tw1, tid, nthr);
+      __syncthreads();
+      if (x < nh) {
+        const int k = x;
+#pragma unroll
+        for (int q = 0; q < NSF; ++q) {
+          const C Zk = fbuf[q * rpitch(n1) + rpad(k)];
+          const C Zn = fbuf[q * rpitch(n1) + rpad(k == 0 ? 0 : n1 - k)];
+          C A, B;
+          A.x = T(0.5) * (Zk.x + Zn.x);
+          A.y = T(0.5) * (Zk.y - Zn.y);
+          B.x = T(0.5) * (Zk.y + Zn.y);
+          B.y = T(0.5) * (Zn.x - Zk.x);
+          const int ra = 2 * q;
+          const int c = ra / TY, r = ra - c * TY;
+          const size_t o = c * comp_stride + (size_t)zp * plane_stride + (size_t)(y0 + r) * P + k;
+          out[o] = A;
+          out[o + P] = B;
         }
       }
     }
@@ -719,7 +633,7 @@ __global__ void __launch_bounds__((sizeof(T) == 8 && TY == 8) ? 256 : 512) k_mar
       for (int k = 0; k < 3; ++k) { Fp[r][k] = Fn[r][k]; Fn[r][k] = 0; }
   }
   cp_async_wait_all();
-  if (!FORCE_LIKE) return;
+  if (MODE != MODE_FORCE) return;
   double acc[NRED];
 #pragma unroll
   for (int i = 0; i < 6; ++i) acc[i] = (double)sacc[i];

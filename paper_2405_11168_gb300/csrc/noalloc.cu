@@ -20,14 +20,14 @@
 #include <mutex>
 
 #include "../../include/hs.h"
-#include "launch.h"
+#include "tiling.h"
 
 namespace {
 
 // Layout of the scratch array: status record | phase table | block partials.
 constexpr size_t kStatusBytes = 256;
-constexpr size_t kTableBytes = (size_t)HS_NOALLOC_MAX_PHASES * 21 * sizeof(double);
-constexpr size_t kPartialBytes = (size_t)HS_NOALLOC_MAX_BLOCKS * hs::NRED * sizeof(double);
+constexpr size_t kTableBytes = (size_t)HS_NOALLOC_MAX_PHASES * hs::kAnisoStride<double> * sizeof(double);
+constexpr size_t kPartialBytes = (size_t)HS_NOALLOC_MAX_BLOCKS * hs::kPartStride * sizeof(double);
 constexpr size_t kScratchBytes = kStatusBytes + kTableBytes + kPartialBytes;
 static_assert(kScratchBytes <= HS_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds the stated size");
 // The last int of the status block receives the largest phase id of the call.
@@ -98,28 +98,15 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
     if (!std::isfinite(E[i])) return HS_ERR_INVALID_ARG;
   const int n1 = grid[0], n2 = grid[1], n3 = grid[2];
   const int nthr = ((n1 + 31) / 32) * 32;
-  // rows per block: 4 where N2 allows, halved while the plane ring does not fit
-  // in the device's opt-in shared memory (N1 = 512 needs 2)
-  int dev = 0, smem_optin = 0;
+  int dev = 0, smem_optin = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+      cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return HS_ERR_CUDA;
-  int ty = (n2 % 4 == 0) ? 4 : 2;
-  size_t smem = hs::march_layout(n1, 0, nthr, ty, hs::MODE_FORCE, true, false, 8).total;
-  while (ty > 2 && smem > (size_t)smem_optin) {
-    ty /= 2;
-    smem = hs::march_layout(n1, 0, nthr, ty, hs::MODE_FORCE, true, false, 8).total;
-  }
-  if (smem > (size_t)smem_optin) return HS_ERR_UNSUPPORTED_SIZE;
-  const int ytiles = n2 / ty;
-  int nzc = std::max(1, std::min(n3, (608 + ytiles - 1) / ytiles));
-  const int zc = (n3 + nzc - 1) / nzc;
-  nzc = (n3 + zc - 1) / zc;
-  if ((size_t)ytiles * nzc > (size_t)HS_NOALLOC_MAX_BLOCKS) return HS_ERR_UNSUPPORTED_SIZE;
 
   // phase table in the kernel's layout
   bool iso = true;
-  static thread_local double packed[(size_t)HS_NOALLOC_MAX_PHASES * 21];
+  static thread_local double packed[(size_t)HS_NOALLOC_MAX_PHASES * hs::kAnisoStride<double>];
   for (int p = 0; p < nphase; ++p) {
     double lam, mu;
     if (!isotropic(table + (size_t)p * 36, &lam, &mu)) iso = false;
@@ -131,14 +118,19 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
     if (iso) {
       double lam, mu;
       isotropic(C, &lam, &mu);
-      packed[2 * p] = lam;
-      packed[2 * p + 1] = mu;
+      hs::pack_iso(lam, mu, packed + (size_t)p * hs::kIsoStride<double>);
     } else {
-      int k = 0;
-      for (int i = 0; i < 6; ++i)
-        for (int j = i; j < 6; ++j) packed[(size_t)p * 21 + k++] = C[i * 6 + j];
+      hs::pack_upper(C, packed + (size_t)p * hs::kAnisoStride<double>);
     }
   }
+
+  // rows per block and z chunk: as the FP64 sweeps of hs_solve, within the partial sums the array holds
+  int ty = 2, zc = 1;
+  hs::pick_tile64(iso, n1, n2, n3, 0, (size_t)smem_optin, std::max(1, nsm), HS_NOALLOC_MAX_BLOCKS, &ty, &zc);
+  const size_t smem = hs::real_bytes(true, n1, ty, false);
+  if (smem > (size_t)smem_optin) return HS_ERR_UNSUPPORTED_SIZE;
+  const int ytiles = n2 / ty, nzc = (n3 + zc - 1) / zc;
+  if ((size_t)ytiles * nzc > (size_t)HS_NOALLOC_MAX_BLOCKS) return HS_ERR_UNSUPPORTED_SIZE;
 
   unsigned char* base = nullptr;
   cudaError_t e = scratch_address(&base);
@@ -165,7 +157,7 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
   memcpy(head, &h, sizeof(h));
   e = cudaMemcpyAsync(base, head, kStatusBytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(mat, packed, (size_t)nphase * (iso ? 2 : 21) * sizeof(double), cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(mat, packed, (size_t)nphase * (iso ? hs::kIsoStride<double> : hs::kAnisoStride<double>) * sizeof(double), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return HS_ERR_CUDA;
   // Every id must index the table: the stress kernel reads the table at the
   // id without a bound, so an id >= nphase is refused before it runs.
@@ -193,7 +185,10 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
   a.fout = force;
   a.fout_f32 = 1;
   a.skip_if_done = 0;
-  e = hs::launch_march<double>(a, iso, ty, hs::MODE_FORCE, true, dim3(ytiles, nzc), nthr, smem, s);
+  a.xp = hs::real_pitch(true, ty, hs::MODE_FORCE, n1);
+  // bulk copies need rows that start and end on 16 bytes; the caller's pointers may not
+  a.bulk = (n1 % 8 == 0 && reinterpret_cast<uintptr_t>(u) % 16 == 0 && reinterpret_cast<uintptr_t>(ids) % 16 == 0) ? 1 : 0;
+  e = hs::launch_real<double>(a, iso, ty, hs::MODE_FORCE, dim3(ytiles, nzc), nthr, smem, s);
   if (e != cudaSuccess) return HS_ERR_CUDA;
   e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -32,6 +32,11 @@ template <typename T> struct RowArgs {
   DevStatus* st;
   int skip_if_done;
   size_t zstride;     // batched launches: bytes between the workspaces of consecutive items
+  // R2C, nparts > 0: block 0 sums the partials that the real-space pass left and takes the stopping
+  // test instead of rows; the other blocks share the rows
+  const double* partials;
+  int nparts;
+  double* hist;
 };
 
 template <typename T> __device__ __forceinline__ RowArgs<T> row_item_args(const RowArgs<T>& a) {
@@ -45,6 +50,8 @@ template <typename T> __device__ __forceinline__ RowArgs<T> row_item_args(const 
   b.acc64 = zshift(a.acc64, o);
   b.tw = zshift(a.tw, o);
   b.st = zshift(a.st, o);
+  b.partials = zshift(a.partials, o);
+  b.hist = zshift(a.hist, o);
   return b;
 }
 
@@ -117,7 +124,7 @@ __device__ __forceinline__ void row_stage(const RowArgs<T>& a, const RowLayout& 
   cp_async_commit();
 }
 
-// Persistent: block j transforms batches j, j + gridDim.x, ...; the copy of the
+// Persistent: block j of nblk transforms batches j, j + nblk, ...; the copy of the
 // next batch runs while the current one is transformed.
 // LF > 0: N1 = LF and 256 threads per block, fixed at compile time (hot
 // sizes); LF = 0: both taken at run time; LF = -1: run time, plans with a
@@ -127,8 +134,21 @@ template <typename T, int MODE, int LF = 0, bool BATCH = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowArgs<T> a_) {
   using C = typename cplx_t<T>::type;
   const RowArgs<T> a = BATCH ? row_item_args(a_) : a_;
-  if (a.st->retired || (a.skip_if_done && a.st->done)) return;
+  // In the pass that takes the stopping test the done flag may change while blocks start: the block
+  // decides as one.
+  bool skip = a.st->retired || (a.skip_if_done && a.st->done);
+  if (MODE == ROW_R2C) skip = __syncthreads_or(skip);
+  if (skip) return;
   extern __shared__ __align__(16) unsigned char smraw[];
+  // The stopping test of this evaluation runs beside the row transforms instead of at the end of the
+  // real-space pass, where the whole chip waited for one block (12 of 31 us at 64^3).  A done flag
+  // that it sets is seen by the next kernels; blocks of this one that see it early skip rows nobody reads.
+  const int nfin = (MODE == ROW_R2C && a.nparts > 0) ? 1 : 0;
+  if (MODE == ROW_R2C && nfin && blockIdx.x == 0) {
+    finalize_partials(a.nparts, a.partials, a.st, a.hist, reinterpret_cast<double*>(smraw));
+    return;
+  }
+  const int blk = (int)blockIdx.x - nfin, nblk = (int)gridDim.x - nfin;
   const int n1 = LF > 0 ? LF : a.n1, P = a.P, nh = n1 / 2 + 1, half = n1 / 2;
   const int tid = threadIdx.x, nthr = LF > 0 ? 256 : (int)blockDim.x;
   const RowLayout L = row_layout(MODE, n1, P, nthr, (int)sizeof(T));
@@ -178,15 +198,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowAr
   C* const tws = reinterpret_cast<C*>(smraw + L.tws);
   if constexpr (LF > 0) stage_twiddles<LF>(tws, a.tw, tid, nthr);
   int buf = 0;
-  if ((int)blockIdx.x < nbatch && (!bload || tid == 0)) row_stage<T, MODE>(a, L, smraw, blockIdx.x, 0, bload);
+  if (blk < nbatch && (!bload || tid == 0)) row_stage<T, MODE>(a, L, smraw, blk, 0, bload);
   int k = 0;
-  for (int b = blockIdx.x; b < nbatch; b += gridDim.x, buf ^= 1, ++k) {
+  for (int b = blk; b < nbatch; b += nblk, buf ^= 1, ++k) {
     if (bload) timed_out |= !mbar_wait(sbar + buf, (unsigned)((k >> 1) & 1));
     else cp_async_wait_all();
     if (bulk && tid == 0) bulk_wait_read_all();  // staging buffer buf ^ 1 is free again
     __syncthreads();
-    if (b + (int)gridDim.x < nbatch && (!bload || tid == 0))
-      row_stage<T, MODE>(a, L, smraw, b + gridDim.x, buf ^ 1, bload);
+    if (b + nblk < nbatch && (!bload || tid == 0)) row_stage<T, MODE>(a, L, smraw, b + nblk, buf ^ 1, bload);
     unsigned char* stg = smraw + L.zbytes + (size_t)buf * L.stage;
     const size_t nr = min((size_t)2 * G, (size_t)a.nrows - 2 * (size_t)b * G);
     const int s = b * G + grp;
@@ -350,7 +369,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowAr
   }
   cp_async_wait_all();
   if (bulk && tid == 0) bulk_wait_all();
-  if (timed_out) a.st->done = DONE_TIMEOUT;
+  if (timed_out) atomicMax(&a.st->done, (int)DONE_TIMEOUT);
 }
 
 }  // namespace hs
