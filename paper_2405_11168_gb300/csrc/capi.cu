@@ -255,6 +255,7 @@ struct hs_ctx {
   bool zstate_smem = false;  // the z pass copies the state tile to shared memory
   // persistent double-buffered y / z passes (k_colp): blocks and shared memory
   bool pipe_y = false, pipe_z = false;
+  bool fixed_y = false, fixed_z = false;  // the y / z passes run a compile-time plan
   // column passes fed by tensor copies: the tile map of work buffer B[b] for the y (axis 0)
   // and z (axis 1) passes, cached with the base, item stride and item count it was made for
   CUtensorMap tmap[2][2];
@@ -707,7 +708,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
 
 // The tensor map of the column-pass tiles of B[b] (see ColArgs::tmap): T elements of the half
 // spectrum as (2P x-values, 3 components, n2, n3, items) with the components' stride inside y,
-// box (2 ct, 3, min(n2, 256), 1, 1) for the y passes (zax = 0) or (2 ct, 3, 1, min(n3, 256), 1)
+// box (2 ct, 3, tile_box(n2), 1, 1) for the y passes (zax = 0) or (2 ct, 3, 1, tile_box(n3), 1)
 // for the z pass (zax = 1).  Made once per buffer, base and batch shape.  False when the driver
 // offers no encoder or refuses the map; the caller then copies with cp.async.
 bool tile_map(hs_ctx* c, int zax, int b, CUtensorMap* out) {
@@ -724,11 +725,11 @@ bool tile_map(hs_ctx* c, int zax, int b, CUtensorMap* out) {
     const int L = zax ? c->n3 : c->n2;
     const cuuint64_t dims[5] = {(cuuint64_t)2 * c->P, 3, (cuuint64_t)c->n2, (cuuint64_t)c->n3, (cuuint64_t)n};
     const cuuint64_t strides[4] = {comp, row, plane, c->batch_stride != 0 ? c->batch_stride : 3 * comp};
-    const cuuint32_t box[5] = {(cuuint32_t)(2 * c->ct), 3, zax ? 1u : (cuuint32_t)std::min(L, 256),
-                               zax ? (cuuint32_t)std::min(L, 256) : 1u, 1};
+    const cuuint32_t box[5] = {(cuuint32_t)(2 * c->ct), 3, zax ? 1u : (cuuint32_t)hs::tile_box(L),
+                               zax ? (cuuint32_t)hs::tile_box(L) : 1u, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     const bool aligned = ((uintptr_t)base % 16 == 0) && (2 * c->ct * (cs / 2)) % 16 == 0 && row % 16 == 0 &&
-                         (c->batch_stride % 16 == 0) && (L <= 256 || L % 256 == 0);
+                         (c->batch_stride % 16 == 0);
     if (enc != nullptr && aligned &&
         enc(&c->tmap[zax][b], c->f64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5,
             const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -740,12 +741,11 @@ bool tile_map(hs_ctx* c, int zax, int b, CUtensorMap* out) {
   return c->tmap_ok[zax][b];
 }
 
-// ColArgs of a column pass over B[b] (zax: 0 = y passes, only where they run persistent; 1 = z
-// pass, one tile per block with the state read point by point): tensor copies where the option
-// and the map allow
+// ColArgs of a column pass over B[b] (zax: 0 = y passes, 1 = z pass with the state read point by point;
+// both at lengths with a compile-time plan): tensor copies where the option and the map allow
 template <typename T> hs_status set_tile_map(hs_ctx* c, hs::ColArgs<T>& a, int zax, int b) {
   a.tma = 0;
-  const bool applies = zax == 0 ? c->pipe_y : !c->zstate_smem;
+  const bool applies = zax == 0 ? c->fixed_y : c->fixed_z && !c->zstate_smem;
   if (!applies || c->opt.col_copy == 1) return HS_OK;
   if (tile_map(c, zax, b, &a.tmap)) {
     a.tma = 1;
@@ -1392,12 +1392,18 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
     if (o.col_threads > 0) n = std::max(T, (o.col_threads / T) * T);
     return n;
   };
-  c->nthr_y = col_threads(c->n2);
-  c->nthr_z = col_threads(c->n3);
+  // compile-time plans: the default tile in the plan's block
+  auto col_fixed = [&](int L, int* nthr) {
+    const int nt = hs::col_block(hs::fft_threads<hs::ColPlan>(L), 3 * c->ct, c->f64);
+    const bool fixed = hs::fft_fixed_length(L) && c->ct == (c->f64 ? 4 : 8) && (o.col_threads == 0 || o.col_threads == nt);
+    *nthr = fixed ? nt : col_threads(L);
+    return fixed;
+  };
+  c->fixed_y = col_fixed(c->n2, &c->nthr_y);
+  c->fixed_z = col_fixed(c->n3, &c->nthr_z);
   const size_t cs = c->f64 ? 16 : 8;
-  // a tile, then (fixed lengths) the twiddle table 16 bytes behind it
-  c->smem_y = (size_t)c->n2 * 3 * c->ct * cs + 16 + (size_t)c->n2 * cs;
-  // the z pass may load its tile by a tensor copy: room for its alignment and barrier
+  // a tile, room for a tensor copy's alignment and barrier, then (fixed lengths) the twiddle tables
+  c->smem_y = (size_t)c->n2 * 3 * c->ct * cs + hs::kColpTmaSlack + (size_t)c->n2 * cs;
   c->smem_z = (size_t)c->n3 * 3 * c->ct * cs + hs::kColpTmaSlack + 2 * (size_t)c->n3 * cs;
   c->xfuse = (o.xfuse == 1);
   {
@@ -1476,8 +1482,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
   // persistent row passes: as many blocks as stay resident, at most one per batch
   {
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int T8 = (c->n1 + hs::kE - 1) / hs::kE;
-    const size_t G = (size_t)(c->nthr_row / T8);
+    const size_t G = (size_t)(c->nthr_row / hs::fft_threads<hs::RowPlan>(c->n1));
     const size_t nbatch = ((size_t)3 * c->n2 * c->n3 / 2 + G - 1) / G;
     for (int m = 0; m < 2 && e == cudaSuccess; ++m) {
       int per_sm = 0;
@@ -1504,7 +1509,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
     // 0.247 ms; the y passes gain, 0.095 against 0.101 ms)
     for (int axis = 1; axis <= (o.col_pipe == 2 ? 2 : 1) && o.col_pipe != 1 && !ext && nsm > 0; ++axis) {
       const int L = axis == 1 ? c->n2 : c->n3;
-      if (L != 128 && L != 256 && L != 512) continue;
+      if (!(axis == 1 ? c->fixed_y : c->fixed_z) || L < 128) continue;
       if (axis == 2 && c->zstate_smem) continue;  // the persistent z pass reads the state point by point
       // the tiles may arrive by tensor copies: room for their alignment and barriers
       // and for the twiddle tables behind them

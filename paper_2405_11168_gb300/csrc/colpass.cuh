@@ -26,6 +26,8 @@ enum { COL_Y_FWD = 0, COL_Y_INV = 1, COL_Z_GREEN = 2, COL_Z_INV_STATE = 3 };
 // dynamic shared memory a TMA-fed persistent column pass needs beyond its two tiles (alignment
 // of the tiles to 128 bytes, two mbarriers)
 constexpr size_t kColpTmaSlack = 256;
+// rows of a tile that one tensor copy brings (boxes have at most 256)
+__host__ __device__ constexpr int tile_box(int L) { return L <= 256 ? L : L / 2; }
 
 template <typename T> struct ColArgs {
   using C = typename cplx_t<T>::type;
@@ -52,7 +54,7 @@ template <typename T> struct ColArgs {
   int tma;           // persistent y passes and the fixed-length z pass: tiles loaded by tensor
                      // copies described by tmap
   // rank-5 tiled map of buf as T elements: (2P x-values, 3 components, n2, n3, items), box
-  // (2 CT, 3, min(n2, 256), 1, 1) for the y passes or (2 CT, 3, 1, min(n3, 256), 1) for the z
+  // (2 CT, 3, tile_box(n2), 1, 1) for the y passes or (2 CT, 3, 1, tile_box(n3), 1) for the z
   // pass; the component dimension sits inside y so that a box lands as the [e][comp][col] tile
   CUtensorMap tmap;
 };
@@ -217,7 +219,7 @@ __device__ __forceinline__ void col_green(const ColArgs<T>& a, typename cplx_t<T
   }
 }
 
-// col_green for a compile-time length L and block size NT (NT a multiple of CT): thread tid keeps
+// col_green for a compile-time length L and block size NT (a multiple of CT): thread tid keeps
 // column tid % CT and walks z = tid / CT, tid / CT + NT / CT, ..., so exp(-i q_x), its product
 // with the block's exp(-i q_y), the state address of its column and whether its (q_x, q_y) can
 // be a translation mode are set once; per point only exp(-i q_z) and two products remain.
@@ -228,14 +230,14 @@ __device__ __forceinline__ void col_green_fixed(const ColArgs<T>& a, typename cp
                                                 size_t rstride, size_t cstride, int x0, int outer, int ncol,
                                                 int tid, const typename cplx_t<T>::type* tz) {
   using C = typename cplx_t<T>::type;
-  static_assert(NT % CT == 0 && (L * CT) % NT == 0, "whole columns per thread");
+  static_assert(NT % CT == 0, "a column per thread");
   constexpr int W = 3 * CT;
   constexpr int ZS = NT / CT;        // z step of a thread
-  constexpr int NPT = L * CT / NT;   // points per thread
+  constexpr int NPT = (L + ZS - 1) / ZS;  // points per thread; the last may lie beyond the column
+  constexpr bool RAGGED = L % ZS != 0;
   // points in groups of GU; the state loads of the next group are issued before the update of
   // the current one (different points), so their latency runs under its arithmetic
   constexpr int GU = NPT < 2 ? NPT : 2;
-  static_assert(NPT % GU == 0, "whole groups per thread");
   const int col = tid % CT, zt = tid / CT;
   if (col >= ncol) return;
   const bool c0iso = a.c0iso || a.c0dev != nullptr;
@@ -250,7 +252,9 @@ __device__ __forceinline__ void col_green_fixed(const ColArgs<T>& a, typename cp
   auto load_group = [&](C (&V)[GU][3], int u0) {
 #pragma unroll
     for (int u = 0; u < GU; ++u) {
-      const size_t g = (size_t)(zt + (u0 + u) * ZS) * rstride;
+      const int z = zt + (u0 + u) * ZS;
+      if ((RAGGED || NPT % GU != 0) && z >= L) continue;
+      const size_t g = (size_t)z * rstride;
 #pragma unroll
       for (int c = 0; c < 3; ++c) V[u][c] = Sc[c * cstride + g];
     }
@@ -268,6 +272,7 @@ __device__ __forceinline__ void col_green_fixed(const ColArgs<T>& a, typename cp
 #pragma unroll
     for (int u = 0; u < GU; ++u) {
       const int z = zt + (u0 + u) * ZS;
+      if ((RAGGED || NPT % GU != 0) && z >= L) continue;
       C F[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) F[c] = sm[z * W + c * CT + col];
@@ -288,16 +293,25 @@ __device__ __forceinline__ void col_green_fixed(const ColArgs<T>& a, typename cp
   }
 }
 
+// register limits of k_col: 768 (FP32) or 384 (FP64) threads per SM, two thirds of that for FP32
+// plans that hold more than 16 values per thread or take a radix-12 stage (128^3 z pass at 768 / 512 threads:
+// 27.5 / 30.7 us; 192^3 with 24 values: 129 / 110)
+__host__ __device__ constexpr int col_max_threads(int nt, bool f64) { return nt > 0 ? nt : f64 ? 384 : 768; }
+__host__ __device__ constexpr int col_min_blocks(int nt, bool f64, bool wide) {
+  return nt > 0 ? (f64 ? 384 : wide ? 512 : 768) / nt : 1;
+}
+
 // LF > 0: the transformed length is LF and the block has NT threads, both
 // fixed at compile time (hot sizes); LF = 0: both taken at run time; LF = -1:
 // run time, plans with a radix-5, 7 or 11 stage.
-// TMA (z pass with the state read point by point, fixed lengths): thread 0 loads the tile by
-// tensor copies (one per 256 planes) on an mbarrier while every thread issues the state's L2
+// TMA (fixed lengths; the z pass with the state read point by point): thread 0 loads the tile by
+// tensor copies (at most 256 rows each) on an mbarrier while every thread issues the state's L2
 // prefetch; the wait is bounded (a timeout is recorded in the status).
 template <typename T, int CT, int MODE, int LF = 0, int NT = 0, bool TMA = false>
-__global__ void __launch_bounds__(sizeof(T) == 8 ? 384 : 768) k_col(const __grid_constant__ ColArgs<T> a_) {
+__global__ void __launch_bounds__(col_max_threads(NT, sizeof(T) == 8), col_min_blocks(NT, sizeof(T) == 8, LF > 0 && fft_very_wide<ColPlan<(LF > 0 ? LF : 64)>>()))
+    k_col(const __grid_constant__ ColArgs<T> a_) {
   using C = typename cplx_t<T>::type;
-  static_assert(!TMA || (MODE == COL_Z_GREEN && LF > 0), "tensor copies: fixed-length z pass");
+  static_assert(!TMA || (MODE != COL_Z_INV_STATE && LF > 0), "tensor copies: fixed lengths, iteration modes");
   const ColArgs<T> a = col_item_args(a_);
   if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -332,7 +346,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 384 : 768) k_col(const __grid
   C* const tzs = tws + L;
   auto copy_tables = [&]() {
     if constexpr (LF > 0) {
-      stage_twiddles<LF>(tws, tw, tid, nthr);
+      stage_twiddles<ColPlan<LF>>(tws, tw, tid, nthr);
       if (MODE == COL_Z_GREEN)
         for (int i = tid; i < L; i += nthr) tzs[i] = __ldg(tw + i);
     }
@@ -349,13 +363,17 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 384 : 768) k_col(const __grid
       mbar_init(tbar, 1);
       mbar_init_fence();
       mbar_arrive_expect_tx(tbar, (unsigned)(L * W * sizeof(C)));
+      constexpr int HB = tile_box(LF);
 #pragma unroll
-      for (int h = 0; h < (L + 255) / 256; ++h)
-        tma_load_5d(sm + (size_t)h * 256 * W, &a_.tmap, 2 * x0, 0, outer, h * 256, (int)blockIdx.z, tbar);
+      for (int h = 0; h < LF / HB; ++h)
+        tma_load_5d(sm + (size_t)h * HB * W, &a_.tmap, 2 * x0, 0, yaxis ? h * HB : outer, yaxis ? outer : h * HB,
+                    (int)blockIdx.z, tbar);
     }
-    for (int i = tid; i < L * 3; i += nthr) {
-      const int e = i / 3, c = i - 3 * e;
-      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(a.S + c * cstride + base + e * rstride));
+    if (MODE == COL_Z_GREEN) {
+      for (int i = tid; i < L * 3; i += nthr) {
+        const int e = i / 3, c = i - 3 * e;
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(a.S + c * cstride + base + e * rstride));
+      }
     }
     copy_tables();
     __syncthreads();  // the barrier is initialised before anyone waits on it
@@ -412,21 +430,21 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 384 : 768) k_col(const __grid
     io.ccols = ccols;
     io.ncol = ncol;
     if (MODE == COL_Z_GREEN) {
-      fft_col_fixed<LF, W, CT, false, false, false, true>(sm, io, tws, tid, nthr);
+      fft_col_fixed<ColPlan<LF>, W, CT, false, false, false, true>(sm, io, tws, tid, nthr);
       if (ss != nullptr) {
         cp_async_wait_all();
         __syncthreads();
       }
-      if constexpr (NT > 0 && NT % CT == 0 && (LF * CT) % NT == 0) {
+      if constexpr (NT > 0 && NT % CT == 0) {
         if (ss == nullptr) col_green_fixed<T, CT, LF, NT>(a, sm, base, rstride, cstride, x0, outer, ncol, tid, tzs);
         else col_green<T, CT>(a, sm, ss, base, rstride, cstride, x0, outer, ncol, L, tid, nthr);
       } else {
         col_green<T, CT>(a, sm, ss, base, rstride, cstride, x0, outer, ncol, L, tid, nthr);
       }
       __syncthreads();
-      fft_col_fixed<LF, W, CT, true, false, true, true>(sm, io, tws, tid, nthr);
+      fft_col_fixed<ColPlan<LF>, W, CT, true, false, true, true>(sm, io, tws, tid, nthr);
     } else {
-      fft_col_fixed<LF, W, CT, MODE == COL_Y_INV || MODE == COL_Z_INV_STATE, false, true, true>(sm, io, tws, tid,
+      fft_col_fixed<ColPlan<LF>, W, CT, MODE == COL_Y_INV || MODE == COL_Z_INV_STATE, false, true, true>(sm, io, tws, tid,
                                                                                             nthr);
     }
     return;
@@ -457,7 +475,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? 384 : 768) k_col(const __grid
 // and copies the next tile into its second buffer while it transforms the current
 // one, so the copies overlap the arithmetic.  Y_FWD, Y_INV and Z_GREEN (state read
 // point by point after an L2 prefetch issued with the tile's copy).
-// TMA (y passes): thread 0 issues each tile as tensor copies (one per 256 rows) completing on the
+// TMA (y passes): thread 0 issues each tile as tensor copies (at most 256 rows each) completing on the
 // tile buffer's mbarrier, every thread waits on it (bounded; a timeout is recorded in the status).
 template <typename T, int CT, int MODE, int LF, int NT, bool TMA = false>
 __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<T> a_) {
@@ -520,17 +538,18 @@ __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<
     const int x0 = (t % xtiles) * CT, outer = t / xtiles;
     C* sm = sm0 + (size_t)b * L * W;
     mbar_arrive_expect_tx(&tbar[b], (unsigned)(L * W * sizeof(C)));
+    constexpr int HB = tile_box(LF);
 #pragma unroll
-    for (int h = 0; h < (L + 255) / 256; ++h) {
-      if (yaxis) tma_load_5d(sm + (size_t)h * 256 * W, &a_.tmap, 2 * x0, 0, h * 256, outer, (int)blockIdx.z, &tbar[b]);
-      else tma_load_5d(sm + (size_t)h * 256 * W, &a_.tmap, 2 * x0, 0, outer, h * 256, (int)blockIdx.z, &tbar[b]);
+    for (int h = 0; h < LF / HB; ++h) {
+      if (yaxis) tma_load_5d(sm + (size_t)h * HB * W, &a_.tmap, 2 * x0, 0, h * HB, outer, (int)blockIdx.z, &tbar[b]);
+      else tma_load_5d(sm + (size_t)h * HB * W, &a_.tmap, 2 * x0, 0, outer, h * HB, (int)blockIdx.z, &tbar[b]);
     }
   };
   // the plan's per-stage twiddle table behind the barriers, then (z pass) a plain copy of the table
   // for the Green step's z phases (read after the first barrier)
   C* const tws = reinterpret_cast<C*>(smb + (size_t)2 * L * W * sizeof(C) + 16);
   C* const tzs = tws + L;
-  stage_twiddles<LF>(tws, a.tw, tid, NT);
+  stage_twiddles<ColPlan<LF>>(tws, a.tw, tid, NT);
   if (MODE == COL_Z_GREEN)
     for (int i = tid; i < L; i += NT) tzs[i] = __ldg(a.tw + i);
   bool timed_out = false;
@@ -571,16 +590,12 @@ __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<
     io.ccols = min(CT, a.P - x0);
     io.ncol = min(CT, a.nh - x0);
     if (MODE == COL_Z_GREEN) {
-      fft_col_fixed<LF, W, CT, false, false, false, true>(sm, io, tws, tid, NT);
-      if constexpr (NT % CT == 0 && (LF * CT) % NT == 0) {
-        col_green_fixed<T, CT, LF, NT>(a, sm, base, rstride, cstride, x0, outer, io.ncol, tid, tzs);
-      } else {
-        col_green<T, CT>(a, sm, nullptr, base, rstride, cstride, x0, outer, io.ncol, L, tid, NT);
-      }
+      fft_col_fixed<ColPlan<LF>, W, CT, false, false, false, true>(sm, io, tws, tid, NT);
+      col_green_fixed<T, CT, LF, NT>(a, sm, base, rstride, cstride, x0, outer, io.ncol, tid, tzs);
       __syncthreads();
-      fft_col_fixed<LF, W, CT, true, false, true, true>(sm, io, tws, tid, NT);
+      fft_col_fixed<ColPlan<LF>, W, CT, true, false, true, true>(sm, io, tws, tid, NT);
     } else {
-      fft_col_fixed<LF, W, CT, MODE == COL_Y_INV, false, true, true>(sm, io, tws, tid, NT);
+      fft_col_fixed<ColPlan<LF>, W, CT, MODE == COL_Y_INV, false, true, true>(sm, io, tws, tid, NT);
     }
     // this tile's shared writes come before the tensor copy that refills the buffer
     if (TMA) fence_async_smem();

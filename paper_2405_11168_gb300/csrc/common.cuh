@@ -111,66 +111,67 @@ template <typename T> struct MatAniso {
 };
 
 // Evaluation of the stopping test from the sums of one residual evaluation
-// (Eqs. L2-norm, tolerance): sums[0..5] = sum over voxels of sigma^T1 + sigma^T2,
-// sums[6] = sum over corners of |F|^2.  Updates the status (error, history,
-// done flag, applied-stress strain update) and clears the arrival counter.
-// One thread calls it.  The status is read in one go, past L1 (other blocks of
-// this launch may have recorded a timeout in it).
-__device__ inline void finalize_eval(DevStatus* st, double* hist, const double* sums) {
+// (Eqs. L2-norm, tolerance), by one warp: lane v holds sums[v], v < 6 the sum over
+// voxels of sigma^T1 + sigma^T2, v = 6 the sum over corners of |F|^2.  Updates the
+// status (error, history, done flag, applied-stress strain update) and clears the
+// arrival counter.  The status is read in one go, past L1 (other blocks of this
+// launch may have recorded a timeout in it).  The divisions and roots run lane by
+// lane: each takes some 25 FP64 instructions, 64 cycles apiece whatever the number
+// of active lanes (one thread took 10 in a row, 8 us of a 13 us pass at 64^3).
+__device__ inline void finalize_eval(DevStatus* st, double* hist, double sum) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
   const int done0 = __ldcg(&st->done), k = __ldcg(&st->evals), max_iter = __ldcg(&st->max_iter),
             hist_cap = __ldcg(&st->hist_cap);
   const double tol = __ldcg(&st->tol), denom = __ldcg(&st->denom), n = __ldcg(&st->nvox),
                rel_tol = __ldcg(&st->rel_tol), err_min0 = __ldcg(&st->err_min), err_first0 = __ldcg(&st->err_first);
   const double* const macro =
       reinterpret_cast<const double*>(__ldcg(reinterpret_cast<const unsigned long long*>(&st->macro)));
-  st->counter = 0;
+  if (lane == 0) st->counter = 0;
   if (done0 == DONE_TIMEOUT || done0 == DONE_FAULT) return;
-  double sm[6], nrm2 = 0;
+  const double mean = (lane < 6 ? 0.5 * sum : sum) / n;  // <sigma> (lanes 0-5), mean |F|^2 (lane 6)
+  double nrm2 = 0;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    sm[i] = 0.5 * sums[i] / n;
-    nrm2 += (i < 3 ? 1.0 : 2.0) * sm[i] * sm[i];
-    st->sig_mean[i] = sm[i];
+    const double m = __shfl_sync(kAll, mean, i);
+    nrm2 += (i < 3 ? 1.0 : 2.0) * m * m;
   }
-  const double l2 = sqrt(sums[6] / n);
-  const double nrm = sqrt(nrm2);
+  const double root = sqrt(lane == 6 ? mean : nrm2);
+  const double l2 = __shfl_sync(kAll, root, 6), nrm = __shfl_sync(kAll, root, 0);
   const double den = denom > 0 ? denom : nrm;
   double err;
   if (den > 0) err = l2 / den;
   else err = (l2 == 0) ? 0.0 : __longlong_as_double(0x7ff0000000000000LL);
-  st->l2 = l2;
-  st->sig_norm = nrm;
-  st->err = err;
-  if (k < hist_cap) hist[k] = err;
-  st->evals = k + 1;
+  if (lane < 6) st->sig_mean[lane] = mean;
   int done = DONE_RUNNING;
-  if (!(err == err) || err > 1e300) {
-    done = DONE_DIVERGED;
-  } else {
-    const double err_min = (k == 0 || err < err_min0) ? err : err_min0;
-    const double err_first = k == 0 ? err : err_first0;
-    st->err_min = err_min;
-    st->err_first = err_first;
-    if (err < tol || (rel_tol > 0 && err <= rel_tol * err_first)) done = DONE_CONVERGED;
-    else if (err > 1e6 * err_min && k > 10) done = DONE_DIVERGED;
-    else if (k + 1 >= max_iter) done = DONE_MAXITER;
+  const bool bad = !(err == err) || err > 1e300;
+  const double err_min = (k == 0 || err < err_min0) ? err : err_min0;
+  const double err_first = k == 0 ? err : err_first0;
+  if (bad) done = DONE_DIVERGED;
+  else if (err < tol || (rel_tol > 0 && err <= rel_tol * err_first)) done = DONE_CONVERGED;
+  else if (err > 1e6 * err_min && k > 10) done = DONE_DIVERGED;
+  else if (k + 1 >= max_iter) done = DONE_MAXITER;
+  if (lane == 0) {
+    st->l2 = l2;
+    st->sig_norm = nrm;
+    st->err = err;
+    if (k < hist_cap) hist[k] = err;
+    st->evals = k + 1;
+    if (!bad) {
+      st->err_min = err_min;
+      st->err_first = err_first;
+    }
+    if (done != DONE_RUNNING) atomicMax(&st->done, done);  // a timeout recorded meanwhile stays
   }
-  if (done != DONE_RUNNING) atomicMax(&st->done, done);  // a timeout recorded meanwhile stays
   if (macro != nullptr && done == DONE_RUNNING) {
     // E <- (lambda0)^-1 : {sigma^a + (lambda0 - <lambda>) : E - <lambda : deps> + <lambda : eps0>}
-    //    = E + (lambda0)^-1 : (sigma^a - <sigma>)   (the same quantity, regrouped)
-    const double* Sa = macro;
-    const double* S0 = macro + 6;
-    double d[6];
+    //    = E + (lambda0)^-1 : (sigma^a - <sigma>)   (the same quantity, regrouped), a component per lane
+    const int i = lane < 6 ? lane : 0;
+    const double d = macro[i] - mean;
+    double acc = 0;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) d[i] = Sa[i] - sm[i];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      double acc = 0;
-#pragma unroll
-      for (int j = 0; j < 6; ++j) acc += S0[i * 6 + j] * d[j];
-      st->E[i] += acc;
-    }
+    for (int j = 0; j < 6; ++j) acc += macro[6 + i * 6 + j] * __shfl_sync(kAll, d, j);
+    if (lane < 6) st->E[lane] += acc;
   }
 }
 
@@ -259,11 +260,7 @@ __device__ inline void finalize_partials(int nblk, const double* partials, DevSt
     }
   }
   const double t = block_sum8(a8, scratch);
-  // the sums of lanes 0..7 to one thread
-  double sums[NRED];
-#pragma unroll
-  for (int v = 0; v < NRED; ++v) sums[v] = __shfl_sync(0xffffffffu, t, v);
-  if (threadIdx.x == 0) finalize_eval(st, hist, sums);
+  if (threadIdx.x < 32) finalize_eval(st, hist, t);
 }
 
 // Publish this block's partials; the last block to arrive takes the sum and the

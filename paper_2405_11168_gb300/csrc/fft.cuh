@@ -131,6 +131,94 @@ template <int A, int B, bool INV, typename C> __device__ __forceinline__ void df
   }
 }
 
+// DFT of length A*B, A and B coprime, without twiddles (prime factor map): n = B n1 + A n2,
+// k = k1 (mod A), k = k2 (mod B).  U = B^-1 mod A, V = A^-1 mod B.
+template <int A, int B, int U, int V, bool INV, typename C> __device__ __forceinline__ void dft_coprime(C* v) {
+  static_assert((B * U) % A == 1 % A && (A * V) % B == 1 % B, "inverse residues");
+  constexpr int N = A * B;
+  C y[B][A];
+#pragma unroll
+  for (int n2 = 0; n2 < B; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < A; ++n1) y[n2][n1] = v[(B * n1 + A * n2) % N];
+    Dft<A, INV, C>::run(y[n2]);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < A; ++k1) {
+    C z[B];
+#pragma unroll
+    for (int n2 = 0; n2 < B; ++n2) z[n2] = y[n2][k1];
+    Dft<B, INV, C>::run(z);
+#pragma unroll
+    for (int k2 = 0; k2 < B; ++k2) v[(B * U * k1 + A * V * k2) % N] = z[k2];
+  }
+}
+template <bool INV, typename C> struct Dft<6, INV, C> {
+  static __device__ __forceinline__ void run(C* v) { dft_coprime<2, 3, 1, 2, INV>(v); }
+};
+template <bool INV, typename C> struct Dft<12, INV, C> {
+  static __device__ __forceinline__ void run(C* v) { dft_coprime<3, 4, 1, 3, INV>(v); }
+};
+
+// cos and sin of 2 pi j / P, 1 <= j <= (P - 1) / 2, for the odd prime radices
+template <int P> __host__ __device__ constexpr double prime_cos(int j) {
+  if (P == 5) return j == 1 ? 0.30901699437494745 : -0.8090169943749473;
+  if (P == 7) return j == 1 ? 0.6234898018587336 : j == 2 ? -0.22252093395631434 : -0.900968867902419;
+  return j == 1 ? 0.8412535328311812 : j == 2 ? 0.41541501300188644 : j == 3 ? -0.142314838273285
+       : j == 4 ? -0.654860733945285 : -0.9594929736144974;
+}
+template <int P> __host__ __device__ constexpr double prime_sin(int j) {
+  if (P == 5) return j == 1 ? 0.9510565162951535 : 0.5877852522924732;
+  if (P == 7) return j == 1 ? 0.7818314824680298 : j == 2 ? 0.9749279121818236 : 0.43388373911755823;
+  return j == 1 ? 0.5406408174555976 : j == 2 ? 0.9096319953545183 : j == 3 ? 0.9898214418809328
+       : j == 4 ? 0.7557495743542583 : 0.28173255684142967;
+}
+// The same at any multiple, folded to the first half turn.
+template <int P> __host__ __device__ constexpr double prime_cos_at(int jk) {
+  const int r = jk % P;
+  return r == 0 ? 1.0 : prime_cos<P>(r <= P / 2 ? r : P - r);
+}
+template <int P> __host__ __device__ constexpr double prime_sin_at(int jk) {
+  const int r = jk % P;
+  return r == 0 ? 0.0 : r <= P / 2 ? prime_sin<P>(r) : -prime_sin<P>(P - r);
+}
+// Odd prime length: sums and differences of the mirrored inputs, then (P - 1) / 2 real combinations for
+// each mirrored pair of outputs, with constant coefficients: (P - 1)^2 multiplications (of reals) where
+// the plain sum takes 4 (P - 1)^2 and reads its coefficients from memory.
+template <int P, bool INV, typename C> struct DftPrime {
+  static __device__ __forceinline__ void run(C* v) {
+    using R = decltype(C::x);
+    constexpr int H = P / 2;
+    C s[H], d[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      s[j] = cadd(v[j + 1], v[P - 1 - j]);
+      d[j] = csub(v[j + 1], v[P - 1 - j]);
+    }
+    const C x0 = v[0];
+    C sum = x0;
+#pragma unroll
+    for (int j = 0; j < H; ++j) sum = cadd(sum, s[j]);
+    v[0] = sum;
+#pragma unroll
+    for (int k = 1; k <= H; ++k) {
+      C a = x0, b = cmk<C>(0, 0);
+#pragma unroll
+      for (int j = 1; j <= H; ++j) {
+        const R c = (R)prime_cos_at<P>(j * k), w = (R)prime_sin_at<P>(j * k);
+        a = cmk<C>(a.x + c * s[j - 1].x, a.y + c * s[j - 1].y);
+        b = cmk<C>(b.x + w * d[j - 1].x, b.y + w * d[j - 1].y);
+      }
+      const C ib = rot90<INV>(b);  // forward: -i b, inverse: i b
+      v[k] = cadd(a, ib);
+      v[P - k] = csub(a, ib);
+    }
+  }
+};
+template <bool INV, typename C> struct Dft<5, INV, C> : DftPrime<5, INV, C> {};
+template <bool INV, typename C> struct Dft<7, INV, C> : DftPrime<7, INV, C> {};
+template <bool INV, typename C> struct Dft<11, INV, C> : DftPrime<11, INV, C> {};
+
 template <bool INV, typename C> struct Dft<8, INV, C> {
   static __device__ __forceinline__ void run(C* v) { dft_composite<2, 4, INV>(v); }
 };
@@ -211,28 +299,11 @@ __device__ __forceinline__ void stockham_stage(C* buf, int ss, int es, int ps, i
         }
       }
       const int base = pq * Ns * R + kk;
-      if constexpr (R == 5 || R == 7 || R == 11) {
-        // table DFT: each output straight to its place (no array of R outputs kept live)
-        const int tstep = L / R;
-#pragma unroll 1
-        for (int q = 0; q < R; ++q) {
-          C acc = v[k][0];
+      Dft<R, INV, C>::run(v[k]);
 #pragma unroll
-          for (int m = 1; m < R; ++m) {
-            C w = __ldg(tw + tstep * ((m * q) % R));
-            if (INV) w.y = -w.y;
-            acc = cadd(acc, cmul(v[k][m], w));
-          }
-          const int e = base + q * Ns;
-          sb[e * es + (ps >= 0 ? (e >> ps) : 0)] = acc;
-        }
-      } else {
-        Dft<R, INV, C>::run(v[k]);
-#pragma unroll
-        for (int m = 0; m < R; ++m) {
-          const int e = base + m * Ns;
-          sb[e * es + (ps >= 0 ? (e >> ps) : 0)] = v[k][m];
-        }
+      for (int m = 0; m < R; ++m) {
+        const int e = base + m * Ns;
+        sb[e * es + (ps >= 0 ? (e >> ps) : 0)] = v[k][m];
       }
     }
   }
@@ -299,46 +370,117 @@ __host__ __device__ inline bool plan_ext(const FftPlan& p) {
 
 
 // ---------------------------------------------------------------------------
-// Compile-time plans for the hot lengths: every stride, stage count and
-// radix is a constant, so the per-element index arithmetic folds away.
+// Compile-time plans: every stride, stage count and radix is a constant, so
+// the per-element index arithmetic folds away.  A plan is its radices and the
+// number of threads T that share a sequence, which divides L / r for every
+// radix r, so that no thread idles in any stage; a thread holds L / T values.
+// Few stages of large radices: a stage costs a load and a store of every value
+// through shared memory and two barriers.  Measured per pass (us, FP32, cubes): columns 128 as 8 x 16 15.5 y
+// and 27.5 z (8 x 4 x 4: 18.8, 38.7), 192 as 8 x 4 x 6 with 8 threads 35, 91 (4 x 4 x 12 with 16: 47, 110;
+// run-time plan 80, 166), 96 as 8 x 12 8.1, 11.0 (4 x 4 x 6: 8.1, 13.0; run-time plan 13, 21), 256 as 8 x 8 x 4
+// 78, 188 (16 x 16: 78, 217); rows 256 as 16 x 16 81 and 73 (8 x 8 x 4: 87, 78), 192 as 4 x 4 x 12 48
+// (8 x 4 x 6: 67; run-time plan 84), 96 as 4 x 4 x 6 10.5 (8 x 12: 11.8), 128 in FP64 as 8 x 4 x 4 158 (8 x 16: 179).
 // ---------------------------------------------------------------------------
-template <int L> struct FixedPlan { static constexpr int n = 0; };
-template <> struct FixedPlan<64> {
-  static constexpr int n = 2;
-  __host__ __device__ static constexpr int r(int i) { return 8; }
+template <int LEN, int THREADS, int NST, int R0, int R1, int R2 = 1, int R3 = 1> struct FixedPlan {
+  static constexpr int L = LEN, n = NST, T = THREADS;
+  __host__ __device__ static constexpr int r(int i) { return i == 0 ? R0 : i == 1 ? R1 : i == 2 ? R2 : R3; }
+  static_assert(R0 * R1 * R2 * R3 == L, "radices");
+  static_assert((L / R0) % T == 0 && (L / R1) % T == 0 && (NST < 3 || (L / R2) % T == 0) && (NST < 4 || (L / R3) % T == 0),
+                "threads");
 };
-template <> struct FixedPlan<128> {
-  static constexpr int n = 3;
-  __host__ __device__ static constexpr int r(int i) { return i == 0 ? 8 : 4; }
-};
-template <> struct FixedPlan<256> {
-  static constexpr int n = 3;
-  __host__ __device__ static constexpr int r(int i) { return i == 2 ? 4 : 8; }
-};
-template <> struct FixedPlan<512> {
-  static constexpr int n = 3;
-  __host__ __device__ static constexpr int r(int i) { return 8; }
-};
+template <int L> struct ColPlan;
+template <> struct ColPlan<32> : FixedPlan<32, 4, 2, 4, 8> {};
+template <> struct ColPlan<48> : FixedPlan<48, 4, 2, 4, 12> {};
+template <> struct ColPlan<64> : FixedPlan<64, 8, 2, 8, 8> {};
+template <> struct ColPlan<96> : FixedPlan<96, 4, 2, 8, 12> {};
+template <> struct ColPlan<128> : FixedPlan<128, 8, 2, 8, 16> {};
+template <> struct ColPlan<192> : FixedPlan<192, 8, 3, 8, 4, 6> {};
+template <> struct ColPlan<256> : FixedPlan<256, 32, 3, 8, 8, 4> {};
+template <> struct ColPlan<384> : FixedPlan<384, 32, 4, 4, 4, 4, 6> {};
+template <> struct ColPlan<512> : FixedPlan<512, 64, 3, 8, 8, 8> {};
+template <int L> struct RowPlan : ColPlan<L> {};
+template <> struct RowPlan<96> : FixedPlan<96, 8, 3, 4, 4, 6> {};
+template <> struct RowPlan<128> : FixedPlan<128, 16, 3, 8, 4, 4> {};
+template <> struct RowPlan<192> : FixedPlan<192, 16, 3, 4, 4, 12> {};
+template <> struct RowPlan<256> : FixedPlan<256, 16, 2, 16, 16> {};
+#define HS_FIXED_LENGTHS(F) F(32) F(48) F(64) F(96) F(128) F(192) F(256) F(384) F(512)
 
-// Position of element e inside a sequence: e*ES + (e >> PS) for PS >= 0, e*ES
-// for PS = -1, and for PS = -2 (rows, ES = 1, length a multiple of 16) the XOR
-// swizzle e ^ (((e >> 2) ^ (e >> 3)) & 15), a permutation of each row that keeps
-// the 64-bit accesses of every stage of the fixed 64..512 plans within 3% of
-// conflict-free (rows of length 64 are spaced 72 apart; see rowpass.cuh).
-template <int ES, int PS> __host__ __device__ __forceinline__ int seq_pos(int e) {
-  if constexpr (PS == -2) return e ^ (((e >> 2) ^ (e >> 3)) & 15);
-  else return e * ES + (PS >= 0 ? (e >> PS) : 0);
+// lengths whose column passes also run persistent
+#define HS_PERSISTENT_LENGTHS(F) F(128) F(192) F(256) F(384) F(512)
+
+// threads per sequence: the plan's, or one per kE values for the run-time plans
+template <template <int> class PLAN> __host__ __device__ inline int fft_threads(int L) {
+  switch (L) {
+#define HS_CASE(LEN) case LEN: return PLAN<LEN>::T;
+    HS_FIXED_LENGTHS(HS_CASE)
+#undef HS_CASE
+    default: return (L + kE - 1) / kE;
+  }
 }
-__host__ __device__ __forceinline__ int rswz(int e) { return seq_pos<1, -2>(e); }
+__host__ __device__ inline bool fft_fixed_length(int L) {
+  switch (L) {
+#define HS_CASE(LEN) case LEN:
+    HS_FIXED_LENGTHS(HS_CASE)
+#undef HS_CASE
+    return true;
+    default: return false;
+  }
+}
 
-// The row swizzle is linear over XOR (shifts, XOR and masks are), and an index that is a sum of
-// parts with disjoint bits is their XOR, so swz(a + b) = swz(a) ^ swz(b) for such parts: a
-// thread swizzles its own offset once per stage and each element adds one XOR with a constant.
-__host__ __device__ constexpr int swz_c(int e) { return e ^ (((e >> 2) ^ (e >> 3)) & 15); }
 __host__ __device__ constexpr int ilog2_c(int v) { return v <= 1 ? 0 : 1 + ilog2_c(v >> 1); }
-// b = pq NS + kk (kk < NS) -> pq NS R + kk: the bits of b at and above log2 NS move up by log2 R
+
+// values a thread of the plan holds; above 8 the passes ask for fewer resident threads, so that the
+// values, a butterfly's temporaries and its twiddles stay in registers
+template <class PL> __host__ __device__ constexpr bool fft_wide() { return PL::L > 8 * PL::T; }
+// more than 16 values, or radix 12
+template <class PL> __host__ __device__ constexpr bool fft_very_wide() {
+  return PL::L > 16 * PL::T || PL::r(0) == 12 || PL::r(1) == 12 || PL::r(2) == 12 || PL::r(3) == 12;
+}
+
+// Block of a column pass over tiles of W sequences: the most sequences at a time that divide W (no thread
+// idles in any round) and stay within 256 (FP32) or 192 (FP64) threads.
+__host__ __device__ constexpr int col_block(int T, int W, bool f64) {
+  const int limit = f64 ? 192 : 256;
+  int g = W;
+  while (g > 1 && (W % g != 0 || g * T > limit)) --g;
+  return (g * T + 31) / 32 * 32;
+}
+
+// Position of element e inside a row (sequence with unit element stride) and the spacing of rows in shared
+// memory, chosen so that the 64-bit accesses of a half-warp fall on different banks in every stage:
+//  * 32, 64, 128, 512: the XOR swizzle e ^ (((e >> 2) ^ (e >> 3)) & 15), rows of 32 and 64 spaced 36 and 72
+//    apart; 256: e ^ ((e >> 4) & 15);
+//  * other lengths: one spare slot per T elements (e + e / T, T a power of two), rows spaced by T (mod 16).
+template <int L> struct RowPos {
+  static constexpr bool pow2 = (L & (L - 1)) == 0;
+  static constexpr int T = RowPlan<L>::T;
+  static constexpr int padded = L + L / T;
+  static constexpr int pitch = L == 32 ? 36 : L == 64 ? 72 : pow2 ? L
+                               : padded + (T >= 16 ? 0 : ((T - padded) % 16 + 16) % 16);
+  __host__ __device__ static constexpr int at(int e) {
+    return L == 256 ? e ^ ((e >> 4) & 15)
+         : pow2 ? e ^ (((e >> 2) ^ (e >> 3)) & 15) : e + (e >> ilog2_c(T));
+  }
+};
+__host__ __device__ inline int row_pitch(int L) {
+  switch (L) {
+#define HS_CASE(LEN) case LEN: return RowPos<LEN>::pitch;
+    HS_FIXED_LENGTHS(HS_CASE)
+#undef HS_CASE
+    default: return rpitch(L);
+  }
+}
+// The swizzles are linear over XOR (shifts, XOR and masks are), and an index that is a sum of parts with
+// disjoint bits is their XOR, so at(a + b) = at(a) ^ at(b) for such parts; the padded positions are
+// additive when the second part is a multiple of T and the first below T.  Either way a thread finds its
+// own part once per stage and each element adds a constant.
+template <int L> __device__ __forceinline__ int row_join(int a, int c) {
+  return RowPos<L>::pow2 ? (a ^ c) : (a + c);
+}
+
+// b = pq NS + kk (kk < NS) -> pq NS R + kk
 template <int NS, int R> __device__ __forceinline__ int stockham_out(int b) {
-  return ((b >> ilog2_c(NS)) << (ilog2_c(NS) + ilog2_c(R))) | (b & (NS - 1));
+  return (b / NS) * (NS * R) + b % NS;
 }
 
 // Twiddle table of a fixed plan in shared memory, laid out per stage: stage s (NS_s = r_0 ... r_{s-1}
@@ -346,25 +488,25 @@ template <int NS, int R> __device__ __forceinline__ int stockham_out(int b) {
 // NS_s - r_0 + (m - 1) NS_s + kk.  The lanes of a warp hold consecutive kk, so they read consecutive
 // entries (no bank conflicts); since (R_s - 1) NS_s = NS_{s+1} - NS_s the stages follow each other
 // and the table has L - r_0 entries.
-template <int L, typename C>
+template <class PL, typename C>
 __device__ __forceinline__ void stage_twiddles(C* tab, const C* __restrict__ tw, int tid, int nthr) {
-  constexpr int R0 = FixedPlan<L>::r(0);
+  constexpr int L = PL::L, R0 = PL::r(0);
   for (int j = tid; j < L - R0; j += nthr) {
     int ns = R0, st = 1;
-    while (st + 1 < FixedPlan<L>::n && j >= ns * FixedPlan<L>::r(st) - R0) {
-      ns *= FixedPlan<L>::r(st);
+    while (st + 1 < PL::n && j >= ns * PL::r(st) - R0) {
+      ns *= PL::r(st);
       ++st;
     }
     const int i = j - (ns - R0);
     const int m = i / ns + 1, kk = i - (m - 1) * ns;
-    tab[j] = __ldg(tw + kk * m * (L / (ns * FixedPlan<L>::r(st))));
+    tab[j] = __ldg(tw + kk * m * (L / (ns * PL::r(st))));
   }
 }
 // twiddle m of butterfly kk in the stage with NS and step: from the per-stage table in shared
 // memory (TWS), or from the plain table through the read-only path
-template <bool TWS, int L, int NS, typename C>
+template <bool TWS, class PL, int NS, typename C>
 __device__ __forceinline__ C stage_tw(const C* __restrict__ tw, int m, int kk, int step) {
-  if constexpr (TWS) return tw[(NS - FixedPlan<L>::r(0)) + (m - 1) * NS + kk];
+  if constexpr (TWS) return tw[(NS - PL::r(0)) + (m - 1) * NS + kk];
   else return __ldg(tw + kk * m * step);
 }
 
@@ -378,84 +520,75 @@ template <bool TWS, typename C> __device__ __forceinline__ C tw_load(const C* __
   }
 }
 
-// one stage; sequence s element e at buf[s*SS + seq_pos<ES, PS>(e)]
-template <int L, int R, int NS, int SS, int ES, int PS, bool INV, bool TWS = false, typename C>
+// one stage on rows; element e of sequence s at buf[s * pitch + at(e)]
+template <class PL, int R, int NS, bool INV, bool TWS = false, typename C>
 __device__ __forceinline__ void stage_fixed(C* buf, int s, int t, bool active, const C* __restrict__ tw, bool wsync) {
-  constexpr int T = L / kE;
+  constexpr int L = PL::L, T = PL::T;
+  using P = RowPos<L>;
   constexpr int nb = L / R;
-  constexpr int KB = (nb + T - 1) / T;
+  constexpr int KB = nb / T;
   constexpr int step = L / (NS * R);
-  // swizzled rows (PS = -2): T, nb, NS and R are powers of two and t < T, so the loads' index
-  // b + m nb = t + k T + m nb and the stores' pq NS R + kk + m NS split into disjoint parts
-  constexpr bool XS = (PS == -2) && (T & (T - 1)) == 0 && (nb & (nb - 1)) == 0 && (NS & (NS - 1)) == 0 &&
-                      (R & (R - 1)) == 0;
-  const int tin = XS ? swz_c(t) : 0;
-  const int tout = XS ? swz_c(stockham_out<NS, R>(t)) : 0;
+  // power-of-two lengths: the stores' pq NS R + kk + m NS splits into disjoint parts too
+  const int tin = P::at(t);
+  const int tout = P::pow2 ? P::at(stockham_out<NS, R>(t)) : 0;
   C v[KB][R];
-  C* sb = buf + s * SS;
+  C* sb = buf + s * P::pitch;
+  if (active) {
 #pragma unroll
-  for (int k = 0; k < KB; ++k) {
-    const int b = t + k * T;
-    if (active && b < nb) {
+    for (int k = 0; k < KB; ++k)
 #pragma unroll
-      for (int m = 0; m < R; ++m) {
-        const int e = b + m * nb;
-        if constexpr (XS) v[k][m] = sb[tin ^ swz_c(k * T + m * nb)];
-        else v[k][m] = sb[seq_pos<ES, PS>(e)];
-      }
-    }
+      for (int m = 0; m < R; ++m) v[k][m] = sb[row_join<L>(tin, P::at(k * T + m * nb))];
   }
   if (wsync) __syncwarp(); else __syncthreads();
+  if (active) {
 #pragma unroll
-  for (int k = 0; k < KB; ++k) {
-    const int b = t + k * T;
-    if (active && b < nb) {
-      const int kk = b & (NS - 1);
-      const int pq = b / NS;
+    for (int k = 0; k < KB; ++k) {
+      const int b = t + k * T;
+      const int kk = b % NS;
       if (NS > 1) {
 #pragma unroll
         for (int m = 1; m < R; ++m) {
-          C w = stage_tw<TWS, L, NS>(tw, m, kk, step);
+          C w = stage_tw<TWS, PL, NS>(tw, m, kk, step);
           if (INV) w.y = -w.y;
           v[k][m] = cmul(v[k][m], w);
         }
       }
       Dft<R, INV, C>::run(v[k]);
-      const int base = pq * NS * R + kk;
+      const int base = stockham_out<NS, R>(b);
 #pragma unroll
       for (int m = 0; m < R; ++m) {
-        const int e = base + m * NS;
-        if constexpr (XS) sb[tout ^ swz_c(stockham_out<NS, R>(k * T) + m * NS)] = v[k][m];
-        else sb[seq_pos<ES, PS>(e)] = v[k][m];
+        if constexpr (P::pow2) {
+          sb[tout ^ P::at((k * T / NS) * (NS * R) + (k * T) % NS + m * NS)] = v[k][m];
+        } else {
+          sb[P::at(base + m * NS)] = v[k][m];
+        }
       }
     }
   }
   if (wsync) __syncwarp(); else __syncthreads();
 }
 
-template <int L, int ST, int NS, int SS, int ES, int PS, bool INV, bool TWS = false, typename C>
+template <class PL, int ST, int NS, bool INV, bool TWS = false, typename C>
 __device__ __forceinline__ void stages_fixed(C* buf, int s, int t, bool active, const C* __restrict__ tw,
                                              bool wsync) {
-  if constexpr (ST < FixedPlan<L>::n) {
-    constexpr int R = FixedPlan<L>::r(ST);
-    stage_fixed<L, R, NS, SS, ES, PS, INV, TWS>(buf, s, t, active, tw, wsync);
-    stages_fixed<L, ST + 1, NS * R, SS, ES, PS, INV, TWS>(buf, s, t, active, tw, wsync);
+  if constexpr (ST < PL::n) {
+    constexpr int R = PL::r(ST);
+    stage_fixed<PL, R, NS, INV, TWS>(buf, s, t, active, tw, wsync);
+    stages_fixed<PL, ST + 1, NS * R, INV, TWS>(buf, s, t, active, tw, wsync);
   }
 }
 
-// Same contract as fft_smem with L, the strides and the mapping fixed at compile time.  TWS: tw
+// Row FFTs of a compile-time plan, sequence s by threads s T .. s T + T - 1 (RowPos layout).  TWS: tw
 // points to the plan's per-stage twiddle table in shared memory (stage_twiddles).
-template <int L, bool INV, bool COLMAP, int SS, int ES, int PS, bool TWS = false, typename C>
-__device__ __forceinline__ void fft_fixed(C* buf, int nseq, const C* __restrict__ tw, int tid, int nthreads) {
-  constexpr int T = L / kE;
+template <class PL, bool INV, bool TWS = false, typename C>
+__device__ __forceinline__ void fft_rows_fixed(C* buf, int nseq, const C* __restrict__ tw, int tid, int nthreads) {
+  constexpr int T = PL::T;
   const int G = nthreads / T;
-  const bool wsync = !COLMAP && T <= 32 && (32 % T) == 0 && (nthreads % 32) == 0;
+  const bool wsync = T <= 32 && (32 % T) == 0 && (nthreads % 32) == 0;
   for (int g0 = 0; g0 < nseq; g0 += G) {
-    const int sl = COLMAP ? (tid % G) : (tid / T);
-    const int t = COLMAP ? (tid / G) : (tid % T);
+    const int sl = tid / T, t = tid % T;
     const int s = g0 + sl;
-    const bool active = (COLMAP ? (t < T) : (sl < G)) && s < nseq;
-    stages_fixed<L, 0, 1, SS, ES, PS, INV, TWS>(buf, s, t, active, tw, wsync);
+    stages_fixed<PL, 0, 1, INV, TWS>(buf, s, t, sl < G && s < nseq, tw, wsync);
   }
 }
 
@@ -467,7 +600,7 @@ __device__ __forceinline__ void fft_fixed(C* buf, int nseq, const C* __restrict_
 // and at sm[e * W + s] in the shared tile.  IN_G: the first stage reads its
 // butterfly inputs from global memory (columns >= ccols read as zero); OUT_G:
 // the last stage writes its outputs to global memory (columns < ncol only).
-// Every other stage goes through the shared tile as in fft_fixed (COLMAP).
+// Every other stage goes through the shared tile.
 // ---------------------------------------------------------------------------
 template <typename C> struct ColIO {
   const C* gin;
@@ -476,19 +609,19 @@ template <typename C> struct ColIO {
   int ccols, ncol;
 };
 
-template <int L, int R, int NS, int W, int CT, bool INV, bool FROM_G, bool TO_G, bool TWS = false, typename C>
+template <class PL, int R, int NS, int W, int CT, bool INV, bool FROM_G, bool TO_G, bool TWS = false, typename C>
 __device__ __forceinline__ void stage_col(C* sm, const ColIO<C>& io, int s, int t, bool active,
                                           const C* __restrict__ tw) {
-  constexpr int T = L / kE;
+  constexpr int L = PL::L, T = PL::T;
   constexpr int nb = L / R;
-  constexpr int KB = (nb + T - 1) / T;
+  constexpr int KB = nb / T;
   constexpr int step = L / (NS * R);
   const int c = s / CT, col = s - c * CT;
   C v[KB][R];
 #pragma unroll
   for (int k = 0; k < KB; ++k) {
     const int b = t + k * T;
-    if (active && b < nb) {
+    if (active) {
       if (FROM_G) {
         const C* gp = io.gin + c * io.cstride + col;
         const bool ok = col < io.ccols;
@@ -507,19 +640,18 @@ __device__ __forceinline__ void stage_col(C* sm, const ColIO<C>& io, int s, int 
 #pragma unroll
   for (int k = 0; k < KB; ++k) {
     const int b = t + k * T;
-    if (active && b < nb) {
-      const int kk = b & (NS - 1);
-      const int pq = b / NS;
+    if (active) {
+      const int kk = b % NS;
       if (NS > 1) {
 #pragma unroll
         for (int m = 1; m < R; ++m) {
-          C w = stage_tw<TWS, L, NS>(tw, m, kk, step);
+          C w = stage_tw<TWS, PL, NS>(tw, m, kk, step);
           if (INV) w.y = -w.y;
           v[k][m] = cmul(v[k][m], w);
         }
       }
       Dft<R, INV, C>::run(v[k]);
-      const int base = pq * NS * R + kk;
+      const int base = stockham_out<NS, R>(b);
       if (TO_G) {
         if (col < io.ncol) {
           C* gp = io.gout + c * io.cstride + col;
@@ -535,29 +667,29 @@ __device__ __forceinline__ void stage_col(C* sm, const ColIO<C>& io, int s, int 
   if (!TO_G) __syncthreads();
 }
 
-template <int L, int ST, int NS, int W, int CT, bool INV, bool IN_G, bool OUT_G, bool TWS = false, typename C>
+template <class PL, int ST, int NS, int W, int CT, bool INV, bool IN_G, bool OUT_G, bool TWS = false, typename C>
 __device__ __forceinline__ void stages_col(C* sm, const ColIO<C>& io, int s, int t, bool active,
                                            const C* __restrict__ tw) {
-  if constexpr (ST < FixedPlan<L>::n) {
-    constexpr int R = FixedPlan<L>::r(ST);
-    constexpr bool FIRST = (ST == 0), LAST = (ST + 1 == FixedPlan<L>::n);
-    stage_col<L, R, NS, W, CT, INV, IN_G && FIRST, OUT_G && LAST, TWS>(sm, io, s, t, active, tw);
-    stages_col<L, ST + 1, NS * R, W, CT, INV, IN_G, OUT_G, TWS>(sm, io, s, t, active, tw);
+  if constexpr (ST < PL::n) {
+    constexpr int R = PL::r(ST);
+    constexpr bool FIRST = (ST == 0), LAST = (ST + 1 == PL::n);
+    stage_col<PL, R, NS, W, CT, INV, IN_G && FIRST, OUT_G && LAST, TWS>(sm, io, s, t, active, tw);
+    stages_col<PL, ST + 1, NS * R, W, CT, INV, IN_G, OUT_G, TWS>(sm, io, s, t, active, tw);
   }
 }
 
 // FFT of the W = 3 * CT columns of a tile; lanes walk across columns (COLMAP).
 // TWS: tw points to the plan's per-stage twiddle table in shared memory (stage_twiddles).
-template <int L, int W, int CT, bool INV, bool IN_G, bool OUT_G, bool TWS = false, typename C>
+template <class PL, int W, int CT, bool INV, bool IN_G, bool OUT_G, bool TWS = false, typename C>
 __device__ __forceinline__ void fft_col_fixed(C* sm, const ColIO<C>& io, const C* __restrict__ tw, int tid,
                                               int nthreads) {
-  constexpr int T = L / kE;
+  constexpr int T = PL::T;
   const int G = nthreads / T;
   for (int g0 = 0; g0 < W; g0 += G) {
     const int sl = tid % G, t = tid / G;
     const int s = g0 + sl;
     const bool active = t < T && s < W;
-    stages_col<L, 0, 1, W, CT, INV, IN_G, OUT_G, TWS>(sm, io, s, t, active, tw);
+    stages_col<PL, 0, 1, W, CT, INV, IN_G, OUT_G, TWS>(sm, io, s, t, active, tw);
   }
 }
 

@@ -1,4 +1,3 @@
-// FP32 instantiations of the solver kernels (column tile: 16 complex = 128 B).
+// FP32 fused x pass and state import / export.
 #include "kernels_impl.cuh"
-HS_INSTANTIATE(float, false, 16, 256)
-
+HS_INSTANTIATE(float)

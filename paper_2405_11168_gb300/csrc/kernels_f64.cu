@@ -1,4 +1,3 @@
-// FP64 instantiations of the solver kernels (column tile: 8 complex = 128 B),
-// including the real-space FP64 residual sweep used by the refined mode.
+// FP64 fused x pass and state import / export.
 #include "kernels_impl.cuh"
-HS_INSTANTIATE(double, true, 8, 128)
+HS_INSTANTIATE(double)

@@ -35,8 +35,8 @@ static cudaError_t march_ty(const MarchArgs<T>& a, bool iso, int mode, dim3 g, i
 template <typename T, int CT, int MODE, int LF = 0, int NT = 0>
 static cudaError_t col_one(const ColArgs<T>& a, dim3 g, int nthr, size_t smem, cudaStream_t s) {
   auto k = k_col<T, CT, MODE, LF, NT>;
-  if constexpr (MODE == COL_Z_GREEN && LF > 0) {
-    if (a.tma && !a.state_smem) k = k_col<T, CT, MODE, LF, NT, true>;
+  if constexpr (MODE != COL_Z_INV_STATE && LF > 0) {
+    if (a.tma && !(MODE == COL_Z_GREEN && a.state_smem)) k = k_col<T, CT, MODE, LF, NT, true>;
   }
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
@@ -60,15 +60,18 @@ template <typename T> static int col_length(const ColArgs<T>& a, int mode) {
   return (mode == COL_Y_FWD || mode == COL_Y_INV) ? a.n2 : a.n3;
 }
 
-// compile-time variants for the default tile and block size at the hot lengths
-template <typename T, int CT, int NT>
+// compile-time variants for the default tile and block size at the lengths that have a plan
+template <typename T, int CT>
 static cudaError_t col_dispatch(const ColArgs<T>& a, int mode, dim3 g, int nthr, size_t smem, cudaStream_t s) {
-  const int L = col_length(a, mode);
-  if (nthr == NT) {
-    if (L == 256) return col_ct<T, CT, 256, NT>(a, mode, g, nthr, smem, s);
-    if (L == 512) return col_ct<T, CT, 512, NT>(a, mode, g, nthr, smem, s);
-    if (L == 128) return col_ct<T, CT, 128, NT>(a, mode, g, nthr, smem, s);
-    if (L == 64) return col_ct<T, CT, 64, NT>(a, mode, g, nthr, smem, s);
+  switch (col_length(a, mode)) {
+#define HS_CASE(LEN)                                                                        \
+  case LEN: {                                                                               \
+    constexpr int NT = col_block(ColPlan<LEN>::T, 3 * CT, sizeof(T) == 8);                \
+    if (nthr == NT) return col_ct<T, CT, LEN, NT>(a, mode, g, nthr, smem, s);               \
+    break;                                                                                  \
+  }
+    HS_FIXED_LENGTHS(HS_CASE)
+#undef HS_CASE
   }
   return col_ct<T, CT>(a, mode, g, nthr, smem, s);
 }
@@ -85,8 +88,10 @@ static cudaError_t colp_one(const ColArgs<T>& a, dim3 g, size_t smem, cudaStream
 }
 
 // the persistent column pass at a fixed length: launch it, or (occ) its blocks per SM
-template <typename T, int CT, int NT, int LF>
-static cudaError_t colp_mode(const ColArgs<T>& a, int mode, dim3 g, size_t smem, cudaStream_t s, int* occ) {
+template <typename T, int CT, int LF>
+static cudaError_t colp_mode(const ColArgs<T>& a, int mode, dim3 g, int nthr, size_t smem, cudaStream_t s, int* occ) {
+  constexpr int NT = col_block(ColPlan<LF>::T, 3 * CT, sizeof(T) == 8);
+  if (nthr != NT) return cudaErrorNotSupported;
   switch (mode) {
     case COL_Y_FWD: return colp_one<T, CT, COL_Y_FWD, LF, NT>(a, g, smem, s, occ);
     case COL_Y_INV: return colp_one<T, CT, COL_Y_INV, LF, NT>(a, g, smem, s, occ);
@@ -95,15 +100,13 @@ static cudaError_t colp_mode(const ColArgs<T>& a, int mode, dim3 g, size_t smem,
   }
 }
 
-template <typename T, int CT, int NT>
-static cudaError_t colp_dispatch(const ColArgs<T>& a, int mode, int L, dim3 g, int nthr, size_t smem,
-                                 cudaStream_t s, int* occ) {
-  if (nthr != NT) return cudaErrorNotSupported;
+template <typename T, int CT>
+static cudaError_t colp_dispatch(const ColArgs<T>& a, int mode, int L, dim3 g, int nthr, size_t smem, cudaStream_t s,
+                                 int* occ) {
   switch (L) {
-    case 64: return colp_mode<T, CT, NT, 64>(a, mode, g, smem, s, occ);
-    case 128: return colp_mode<T, CT, NT, 128>(a, mode, g, smem, s, occ);
-    case 256: return colp_mode<T, CT, NT, 256>(a, mode, g, smem, s, occ);
-    case 512: return colp_mode<T, CT, NT, 512>(a, mode, g, smem, s, occ);
+#define HS_CASE(LEN) case LEN: return colp_mode<T, CT, LEN>(a, mode, g, nthr, smem, s, occ);
+    HS_PERSISTENT_LENGTHS(HS_CASE)
+#undef HS_CASE
     default: return cudaErrorNotSupported;
   }
 }
@@ -131,25 +134,26 @@ static cudaError_t row_occ_one(int nthr, size_t smem, int* n) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, nthr, smem);
 }
 
+// compile-time variants for 256-thread blocks at the lengths that have a plan
 template <typename T, int MODE>
 static cudaError_t row_occ(int n1, int nthr, size_t smem, int* n) {
   if (nthr == 256) {
-    if (n1 == 256) return row_occ_one<T, MODE, 256>(nthr, smem, n);
-    if (n1 == 512) return row_occ_one<T, MODE, 512>(nthr, smem, n);
-    if (n1 == 128) return row_occ_one<T, MODE, 128>(nthr, smem, n);
-    if (n1 == 64) return row_occ_one<T, MODE, 64>(nthr, smem, n);
+    switch (n1) {
+#define HS_CASE(LEN) case LEN: return row_occ_one<T, MODE, LEN>(nthr, smem, n);
+      HS_FIXED_LENGTHS(HS_CASE)
+#undef HS_CASE
+    }
   }
   return row_occ_one<T, MODE>(nthr, smem, n);
 }
-
-// compile-time variants for 256-thread blocks at the hot lengths
 template <typename T, int MODE>
 static cudaError_t row_dispatch(const RowArgs<T>& a, dim3 nb, int nthr, size_t smem, cudaStream_t s) {
   if (nthr == 256) {
-    if (a.n1 == 256) return row_one<T, MODE, 256>(a, nb, nthr, smem, s);
-    if (a.n1 == 512) return row_one<T, MODE, 512>(a, nb, nthr, smem, s);
-    if (a.n1 == 128) return row_one<T, MODE, 128>(a, nb, nthr, smem, s);
-    if (a.n1 == 64) return row_one<T, MODE, 64>(a, nb, nthr, smem, s);
+    switch (a.n1) {
+#define HS_CASE(LEN) case LEN: return row_one<T, MODE, LEN>(a, nb, nthr, smem, s);
+      HS_FIXED_LENGTHS(HS_CASE)
+#undef HS_CASE
+    }
   }
   return row_one<T, MODE>(a, nb, nthr, smem, s);
 }
@@ -182,10 +186,9 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
 
 }  // namespace hs
 
-// CT: the wider column tile (CT / 2 is the default); NT: the default
-// column-pass block size, which gets compile-time variants at hot lengths.
-#define HS_INSTANTIATE(T, REALOK, CT, NT)                                                                 \
-  namespace hs {                                                                                         \
+// The fused x pass and the state's import and export.
+#define HS_INSTANTIATE(T) \
+  namespace hs { \
   template <>                                                                                            \
   cudaError_t launch_march<T>(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 grid, int nthr, size_t smem, \
                               cudaStream_t s) {                                                          \
@@ -203,30 +206,56 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
     }                                                                                                    \
   }                                                                                                      \
   template <>                                                                                            \
-  cudaError_t launch_col<T>(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem,      \
-                            cudaStream_t s) {                                                            \
+  cudaError_t launch_state_export<T>(const typename cplx_t<T>::type* S, double2* out, int n2, int n3,     \
+                                     int nh, int P, cudaStream_t s) {                                    \
+    size_t nrows = (size_t)3 * n3 * n2, n = nrows * nh;                                                  \
+    k_state_export<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S, out, nrows, nh, P);                 \
+    return cudaGetLastError();                                                                           \
+  }                                                                                                      \
+  template <>                                                                                            \
+  cudaError_t launch_state_import<T>(const double2* in, typename cplx_t<T>::type* S, int n2, int n3,      \
+                                     int nh, int P, cudaStream_t s) {                                    \
+    size_t nrows = (size_t)3 * n3 * n2, n = nrows * P;                                                   \
+    k_state_import<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, S, nrows, nh, P);                  \
+    return cudaGetLastError();                                                                           \
+  }                                                                                                      \
+  }
+
+// Column passes.  CT: the wider column tile (CT / 2 is the default).
+#define HS_INSTANTIATE_COLS(T, CT) \
+  namespace hs { \
+  template <> \
+  cudaError_t launch_col<T>(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s) { \
     if (a.buf == nullptr || a.tw == nullptr || ((mode == COL_Z_GREEN || mode == COL_Z_INV_STATE) && a.S == nullptr)) \
-      return cudaErrorInvalidValue;                                                                      \
-    if (plan_ext(a.plan)) return launch_col_ext<T>(a, mode, ct, grid, nthr, smem, s);                  \
-    if (ct == (CT)) return col_ct<T, CT>(a, mode, grid, nthr, smem, s);                                  \
-    if (ct == (CT) / 2) return col_dispatch<T, (CT) / 2, NT>(a, mode, grid, nthr, smem, s);              \
-    return cudaErrorInvalidValue;                                                                        \
-  }                                                                                                      \
-  template <>                                                                                            \
-  cudaError_t launch_colp<T>(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem,     \
-                             cudaStream_t s) {                                                           \
-    if (a.buf == nullptr || a.tw == nullptr || (mode == COL_Z_GREEN && a.S == nullptr))                  \
-      return cudaErrorInvalidValue;                                                                      \
-    if (ct != (CT) / 2 || plan_ext(a.plan) || a.state_smem) return cudaErrorNotSupported;               \
-    return colp_dispatch<T, (CT) / 2, NT>(a, mode, col_length(a, mode), grid, nthr, smem, s, nullptr);   \
-  }                                                                                                      \
-  template <>                                                                                            \
-  cudaError_t colp_blocks_per_sm<T>(int mode, int L, int ct, int nthr, size_t smem, int* n) {            \
-    if (ct != (CT) / 2) return cudaErrorNotSupported;                                                    \
-    ColArgs<T> a;                                                                                        \
-    memset(&a, 0, sizeof(a));                                                                            \
-    return colp_dispatch<T, (CT) / 2, NT>(a, mode, L, dim3(1), nthr, smem, nullptr, n);                  \
-  }                                                                                                      \
+      return cudaErrorInvalidValue; \
+    if (plan_ext(a.plan)) return launch_col_ext<T>(a, mode, ct, grid, nthr, smem, s); \
+    if (ct == (CT)) return col_ct<T, CT>(a, mode, grid, nthr, smem, s); \
+    if (ct == (CT) / 2) return col_dispatch<T, (CT) / 2>(a, mode, grid, nthr, smem, s); \
+    return cudaErrorInvalidValue; \
+  } \
+  }
+
+// Persistent column passes (default tile CT).
+#define HS_INSTANTIATE_COLP(T, CT) \
+  namespace hs { \
+  template <> \
+  cudaError_t launch_colp<T>(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s) { \
+    if (a.buf == nullptr || a.tw == nullptr || (mode == COL_Z_GREEN && a.S == nullptr)) return cudaErrorInvalidValue; \
+    if (ct != (CT) || plan_ext(a.plan) || a.state_smem) return cudaErrorNotSupported; \
+    return colp_dispatch<T, CT>(a, mode, col_length(a, mode), grid, nthr, smem, s, nullptr); \
+  } \
+  template <> \
+  cudaError_t colp_blocks_per_sm<T>(int mode, int L, int ct, int nthr, size_t smem, int* n) { \
+    if (ct != (CT)) return cudaErrorNotSupported; \
+    ColArgs<T> a; \
+    memset(&a, 0, sizeof(a)); \
+    return colp_dispatch<T, CT>(a, mode, L, dim3(1), nthr, smem, nullptr, n); \
+  } \
+  }
+
+// Row passes.
+#define HS_INSTANTIATE_ROWS(T) \
+  namespace hs { \
   template <>                                                                                            \
   cudaError_t launch_row<T>(const RowArgs<T>& a, int mode, dim3 nb, int nthr, size_t smem, cudaStream_t s) { \
     if (a.tw == nullptr || (mode == ROW_C2R ? (a.spec_in == nullptr || (a.real_out == nullptr && a.acc64 == nullptr)) \
@@ -240,20 +269,6 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
   cudaError_t row_blocks_per_sm<T>(int mode, int n1, int nthr, size_t smem, int* n) {                     \
     if (n1 % 5 == 0 || n1 % 7 == 0 || n1 % 11 == 0) return row_blocks_per_sm_ext<T>(mode, nthr, smem, n);  \
     return mode == ROW_C2R ? row_occ<T, ROW_C2R>(n1, nthr, smem, n) : row_occ<T, ROW_R2C>(n1, nthr, smem, n); \
-  }                                                                                                      \
-  template <>                                                                                            \
-  cudaError_t launch_state_export<T>(const typename cplx_t<T>::type* S, double2* out, int n2, int n3,     \
-                                     int nh, int P, cudaStream_t s) {                                    \
-    size_t nrows = (size_t)3 * n3 * n2, n = nrows * nh;                                                  \
-    k_state_export<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S, out, nrows, nh, P);                 \
-    return cudaGetLastError();                                                                           \
-  }                                                                                                      \
-  template <>                                                                                            \
-  cudaError_t launch_state_import<T>(const double2* in, typename cplx_t<T>::type* S, int n2, int n3,      \
-                                     int nh, int P, cudaStream_t s) {                                    \
-    size_t nrows = (size_t)3 * n3 * n2, n = nrows * P;                                                   \
-    k_state_import<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, S, nrows, nh, P);                  \
-    return cudaGetLastError();                                                                           \
   }                                                                                                      \
   }
 

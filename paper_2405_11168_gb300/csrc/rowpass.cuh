@@ -8,8 +8,8 @@
 // ROW_R2C: two real rows a, b form Z = a + i b; after the forward FFT
 //   A[k] = (Z[k] + conj Z[N1-k]) / 2 and B[k] = (Z[k] - conj Z[N1-k]) / (2i).
 //
-// A group of T = N1/8 threads owns one pair of rows at a time; for N1 <= 256
-// the group lies inside one warp and needs only warp barriers.  Blocks are
+// A group of T threads (the plan's, or N1/8) owns one pair of rows at a time;
+// where T divides 32 the group lies inside one warp and needs only warp barriers.  Blocks are
 // persistent and stage their next batch of input rows with cp.async while
 // transforming the current one.
 #pragma once
@@ -75,9 +75,8 @@ struct RowLayout {
 };
 __host__ __device__ inline RowLayout row_layout(int mode, int n1, int P, int nthr, int tsize) {
   RowLayout L;
-  const int T8 = (n1 + kE - 1) / kE;
-  L.G = nthr / T8;
-  L.zbytes = (((size_t)L.G * rpitch(n1) * 2 * tsize) + 15) & ~(size_t)15;
+  L.G = nthr / fft_threads<RowPlan>(n1);
+  L.zbytes = (((size_t)L.G * row_pitch(n1) * 2 * tsize) + 15) & ~(size_t)15;
   L.rowbytes = (mode == ROW_C2R) ? (size_t)P * 2 * tsize : (size_t)n1 * tsize;
   L.outbytes = (mode == ROW_C2R) ? (size_t)n1 * tsize : (size_t)P * 2 * tsize;
   const size_t rb = L.rowbytes > L.outbytes ? L.rowbytes : L.outbytes;
@@ -124,6 +123,9 @@ __device__ __forceinline__ void row_stage(const RowArgs<T>& a, const RowLayout& 
   cp_async_commit();
 }
 
+// resident blocks of 256 threads that the registers must allow
+__host__ __device__ constexpr int row_min_blocks(bool f64, bool wide) { return (f64 ? 2 : 3) - (wide ? 1 : 0); }
+
 // Persistent: block j of nblk transforms batches j, j + nblk, ...; the copy of the
 // next batch runs while the current one is transformed.
 // LF > 0: N1 = LF and 256 threads per block, fixed at compile time (hot
@@ -131,7 +133,8 @@ __device__ __forceinline__ void row_stage(const RowArgs<T>& a, const RowLayout& 
 // radix-5, 7 or 11 stage.
 // BATCH: a batched launch (grid.z items); a single solve's launch uses the arguments as they come.
 template <typename T, int MODE, int LF = 0, bool BATCH = false>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowArgs<T> a_) {
+__global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && fft_wide<RowPlan<(LF > 0 ? LF : 64)>>()))
+    k_row(const RowArgs<T> a_) {
   using C = typename cplx_t<T>::type;
   const RowArgs<T> a = BATCH ? row_item_args(a_) : a_;
   // In the pass that takes the stopping test the done flag may change while blocks start: the block
@@ -152,25 +155,24 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowAr
   const int n1 = LF > 0 ? LF : a.n1, P = a.P, nh = n1 / 2 + 1, half = n1 / 2;
   const int tid = threadIdx.x, nthr = LF > 0 ? 256 : (int)blockDim.x;
   const RowLayout L = row_layout(MODE, n1, P, nthr, (int)sizeof(T));
-  const int T8 = (n1 + kE - 1) / kE;          // threads per sequence
+  const int T8 = LF > 0 ? RowPlan<(LF > 0 ? LF : 64)>::T : (n1 + kE - 1) / kE;  // threads per sequence
   const int G = L.G;                           // sequences per batch
   const int grp = tid / T8, t = tid - grp * T8;
   const bool wsync = T8 <= 32 && (32 % T8) == 0;
-  // fixed lengths: XOR-swizzled rows (length-64 rows 72 apart, so that the
-  // four rows a warp transforms fall on different banks); otherwise one spare
-  // slot per 8
-  constexpr int FP = LF == 64 ? 72 : (LF > 0 ? LF : 1);
-  const int pitch = LF > 0 ? FP : rpitch(n1);
+  // fixed lengths: rows in the plan's layout; otherwise one spare slot per 8
+  constexpr int LP = LF > 0 ? LF : 64;
+  using RP = RowPos<LP>;
+  const int pitch = LF > 0 ? RP::pitch : rpitch(n1);
   C* z = reinterpret_cast<C*>(smraw) + (size_t)grp * pitch;
-  auto zi = [](int e) { return LF > 0 ? rswz(e) : rpad(e); };
-  // fixed lengths: the positions of elements t + j T8 and n1 - (t + j T8) from the thread's
-  // swizzled offsets and one XOR with a constant (the swizzle is linear over XOR; see fft.cuh)
-  constexpr int T8C = LF > 0 ? LF / kE : 1;
-  const int tsw = LF > 0 ? rswz(t) : 0;
-  const int tmir = (LF > 0 && t > 0) ? rswz(T8C - t) : 0;
-  auto zfwd = [&](int j) { return LF > 0 ? (tsw ^ swz_c(j * T8C)) : zi(t + j * T8); };
+  auto zi = [](int e) { return LF > 0 ? RP::at(e) : rpad(e); };
+  // fixed lengths: the positions of elements t + j T8 and n1 - (t + j T8) from the thread's own
+  // positions and a constant (see RowPos)
+  constexpr int T8C = RowPlan<LP>::T;
+  const int tsw = RP::at(t);
+  const int tmir = t > 0 ? RP::at(T8C - t) : 0;
+  auto zfwd = [&](int j) { return LF > 0 ? row_join<LP>(tsw, RP::at(j * T8C)) : zi(t + j * T8); };
   auto zmir = [&](int j) {  // position of n1 - (t + j T8), for t + j T8 > 0
-    if (LF > 0) return t == 0 ? swz_c(LF - j * T8C) : (tmir ^ swz_c(LF - (j + 1) * T8C));
+    if (LF > 0) return t == 0 ? RP::at(LP - j * T8C) : row_join<LP>(tmir, RP::at(LP - (j + 1) * T8C));
     return zi(n1 - t - j * T8);
   };
   const int nseq = a.nrows / 2;
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowAr
   // fixed lengths: the transforms read their twiddles from the plan's per-stage table in shared
   // memory (first read after the barrier that opens the first batch)
   C* const tws = reinterpret_cast<C*>(smraw + L.tws);
-  if constexpr (LF > 0) stage_twiddles<LF>(tws, a.tw, tid, nthr);
+  if constexpr (LF > 0) stage_twiddles<RowPlan<LF>>(tws, a.tw, tid, nthr);
   int buf = 0;
   if (blk < nbatch && (!bload || tid == 0)) row_stage<T, MODE>(a, L, smraw, blk, 0, bload);
   int k = 0;
@@ -241,7 +243,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowAr
       }
       group_sync(wsync);
       if constexpr (LF > 0) {
-        fft_fixed<LF, true, false, FP, 1, -2, true>(reinterpret_cast<C*>(smraw), G, tws, tid, nthr);
+        fft_rows_fixed<RowPlan<LF>, true, true>(reinterpret_cast<C*>(smraw), G, tws, tid, nthr);
       } else {
         fft_smem<true, false, (LF < 0)>(reinterpret_cast<C*>(smraw), pitch, 1, 3, G, plan.L, plan.nstage, plan.packed, a.tw,
                               tid, nthr);
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_row(const RowAr
       }
       group_sync(wsync);
       if constexpr (LF > 0) {
-        fft_fixed<LF, false, false, FP, 1, -2, true>(reinterpret_cast<C*>(smraw), G, tws, tid, nthr);
+        fft_rows_fixed<RowPlan<LF>, false, true>(reinterpret_cast<C*>(smraw), G, tws, tid, nthr);
       } else {
         fft_smem<false, false, (LF < 0)>(reinterpret_cast<C*>(smraw), pitch, 1, 3, G, plan.L, plan.nstage, plan.packed, a.tw,
                                tid, nthr);
