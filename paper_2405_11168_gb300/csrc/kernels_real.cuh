@@ -28,9 +28,8 @@ static cudaError_t real_batch(const MarchArgs<T>& a, dim3 g, int nthr, size_t sm
 }
 
 // A launch has a source (correction solves, FP32 force passes only) or an eigenstress, or neither.
-template <typename T, int TY, class MAT, int MODE, int XP, int NT>
+template <typename T, int TY, class MAT, int MODE, int XP, int NT, int B = 0>
 static cudaError_t real_opt(const MarchArgs<T>& a, dim3 g, int nthr, size_t smem, cudaStream_t s, int* occ) {
-  constexpr int B = XP > 0 ? REAL_BULK : 0;
   if (a.src != nullptr) {
     if constexpr (sizeof(T) == 4 && MODE == MODE_FORCE) {
       if (a.sig0 != nullptr) return cudaErrorInvalidValue;
@@ -51,11 +50,16 @@ static cudaError_t real_xp(const MarchArgs<T>& a, dim3 g, int nthr, size_t smem,
     else return cudaErrorInvalidValue;
   } else if constexpr (TY == 4 && MODE == MODE_FORCE) {
     switch (real_pitch_class(false, TY, MODE, a.n1)) {
-      case 64: return real_opt<T, TY, MAT, MODE, 64, 64>(a, g, nthr, smem, s, occ);
-      case 128: return real_opt<T, TY, MAT, MODE, 128, 128>(a, g, nthr, smem, s, occ);
-      case 256: return real_opt<T, TY, MAT, MODE, 256, 256>(a, g, nthr, smem, s, occ);
-      case 512: return real_opt<T, TY, MAT, MODE, 512, 512>(a, g, nthr, smem, s, occ);
-      default: return real_opt<T, TY, MAT, MODE, 0, 512>(a, g, nthr, smem, s, occ);
+#define HS_CASE(P)                                                                                     \
+  case P:                                                                                              \
+    return a.bulk || occ != nullptr ? real_opt<T, TY, MAT, MODE, P, P, REAL_BULK>(a, g, nthr, smem, s, occ) \
+                                    : real_opt<T, TY, MAT, MODE, P, P, 0>(a, g, nthr, smem, s, occ);
+      HS_CASE(64)
+      HS_CASE(128)
+      HS_CASE(256)
+      HS_CASE(512)
+#undef HS_CASE
+      default: return cudaErrorInvalidValue;
     }
   } else {
     return real_opt<T, TY, MAT, MODE, 0, 512>(a, g, nthr, smem, s, occ);

@@ -29,10 +29,10 @@ template <typename T>
 cudaError_t launch_march(const MarchArgs<T>& a, bool iso, int ty, int mode, dim3 grid, int nthr, size_t smem,
                          cudaStream_t s);
 
-// Compile-time row pitch of the pass on a real displacement: the FP32 force pass with tiles of 4 rows and
-// rows that bulk copies take (N1 a multiple of 8) runs the next of four; 0: none.
+// Compile-time row pitch of the pass on a real displacement: the FP32 force pass with tiles of 4 rows runs
+// the next of four; 0: none.
 inline int real_pitch_class(bool f64, int ty, int mode, int n1) {
-  if (f64 || ty != 4 || mode != MODE_FORCE || n1 % 8 != 0) return 0;
+  if (f64 || ty != 4 || mode != MODE_FORCE) return 0;
   return n1 <= 64 ? 64 : n1 <= 128 ? 128 : n1 <= 256 ? 256 : 512;
 }
 // Its row pitch in shared memory.

@@ -217,40 +217,65 @@ __device__ __forceinline__ void real_prefetch_bulk(const MarchArgs<T>& a, const 
   }
 }
 
-// The same plane by every thread, for rows that bulk copies cannot take (a.bulk = 0): 8-byte cp.async
-// of the u and source rows (N1 is even), plain copies of the id rows.  Ends with a commit.
+// Rows of n elements of E bytes by the block's warps, one row per warp and turn: cp.async in the widest chunks
+// (16, 8 or 4 bytes) that start and end every row; 2-byte rows that do not start on 4 bytes element by element.
+// Every thread over every row in turn, 8 bytes at a time, left most of a block without a copy; rows per warp and the
+// compile-time pitch: FP32 force pass 60.8 -> 33.7 us at 100^3, 102 -> 65.7 at 126 x 90 x 210, 254 -> 189
+// at 220 x 200 x 180.
+template <typename E, class Src, class Dst>
+__device__ __forceinline__ void rows_async(int nrows, int n, const Src& src, const Dst& dst) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const unsigned bytes = (unsigned)(n * sizeof(E));
+  for (int r = warp; r < nrows; r += nw) {
+    const unsigned char* const s = reinterpret_cast<const unsigned char*>(src(r));
+    unsigned char* const d = reinterpret_cast<unsigned char*>(dst(r));
+    const unsigned d0 = smem_u32(d), a = bytes | (unsigned)reinterpret_cast<uintptr_t>(s);
+    if ((a & 15) == 0) {
+      for (unsigned q = 16 * lane; q < bytes; q += 512) cp_async16(d + q, s + q);
+    } else if ((a & 7) == 0) {
+      for (unsigned q = 8 * lane; q < bytes; q += 256)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d0 + q), "l"(s + q) : "memory");
+    } else if ((a & 3) == 0) {
+      for (unsigned q = 4 * lane; q < bytes; q += 128)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d0 + q), "l"(s + q) : "memory");
+    } else {
+      for (int q = lane; q < n; q += 32) reinterpret_cast<E*>(d)[q] = reinterpret_cast<const E*>(s)[q];
+    }
+  }
+}
+
+// The same plane by every warp, for rows that bulk copies cannot take (a.bulk = 0).  Ends with a commit.
 template <typename T, int TY>
 __device__ __forceinline__ void real_prefetch_async(const MarchArgs<T>& a, const RealLayout& lay, unsigned char* sm,
                                                     int xp, int y0, int pu, int slot, int ib, int ps, int sb) {
   constexpr int NR = TY + 2;
-  constexpr int EPC = 8 / (int)sizeof(T);
-  const int n1 = a.n1, n2 = a.n2, n3 = a.n3, tid = threadIdx.x, nthr = blockDim.x;
+  const int n1 = a.n1, n2 = a.n2, n3 = a.n3;
   const size_t rplane = (size_t)n2 * n1, rcomp = (size_t)n3 * rplane;
   const int gz = pu < 0 ? pu + n3 : (pu >= n3 ? pu - n3 : pu);
-  auto copy8 = [](void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-  };
   T* const ru = reinterpret_cast<T*>(sm + lay.ring) + (size_t)slot * 3 * NR * xp;
-  for (int r = 0; r < 3 * NR; ++r) {
-    const int c = r / NR, gy = (y0 - 1 + (r - c * NR) + n2) % n2;
-    const T* s = a.ureal + c * rcomp + (size_t)gz * rplane + (size_t)gy * n1;
-    for (int q = tid * EPC; q < n1; q += nthr * EPC) copy8(ru + (size_t)r * xp + q, s + q);
-  }
+  const T* const u = a.ureal + (size_t)gz * rplane;
+  rows_async<T>(3 * NR, n1,
+                [&](int r) {
+                  const int c = r / NR, gy = (y0 - 1 + (r - c * NR) + n2) % n2;
+                  return u + c * rcomp + (size_t)gy * n1;
+                },
+                [&](int r) { return ru + r * xp; });
   if (ib >= 0) {
     uint16_t* const ri = reinterpret_cast<uint16_t*>(sm + lay.ids) + (size_t)ib * (TY + 1) * xp;
-    for (int r = 0; r <= TY; ++r) {
-      const uint16_t* s = a.ids + (size_t)gz * rplane + (size_t)((y0 + r) % n2) * n1;
-      for (int q = tid; q < n1; q += nthr) ri[(size_t)r * xp + q] = s[q];
-    }
+    const uint16_t* const ids = a.ids + (size_t)gz * rplane;
+    rows_async<uint16_t>(TY + 1, n1, [&](int r) { return ids + (size_t)((y0 + r) % n2) * n1; },
+                         [&](int r) { return ri + r * xp; });
   }
   if (sb >= 0) {
     const int zs = ps >= n3 ? ps - n3 : ps;
     float* const rs = reinterpret_cast<float*>(sm + lay.src) + (size_t)sb * 3 * TY * xp;
-    for (int r = 0; r < 3 * TY; ++r) {
-      const int c = r / TY;
-      const float* s = a.src + c * rcomp + (size_t)zs * rplane + (size_t)((y0 + (r - c * TY)) % n2) * n1;
-      for (int q = 2 * tid; q < n1; q += 2 * nthr) copy8(rs + (size_t)r * xp + q, s + q);
-    }
+    const float* const src = a.src + (size_t)zs * rplane;
+    rows_async<float>(3 * TY, n1,
+                      [&](int r) {
+                        const int c = r / TY;
+                        return src + c * rcomp + (size_t)((y0 + (r - c * TY)) % n2) * n1;
+                      },
+                      [&](int r) { return rs + r * xp; });
   }
   cp_async_commit();
 }
@@ -259,7 +284,7 @@ __device__ __forceinline__ void real_prefetch_async(const MarchArgs<T>& a, const
 // XP > 0: compile-time row pitch in shared memory (N1 <= XP), so that row offsets are immediates;
 // XP = 0: a.xp.  NT: the largest block (its registers).  OPT: what the launch has, as compile-time
 // facts (tested at run time they cost a fifth of the instructions: 157.9 against 125.6 M per launch at
-// 256^3, 0.232 against 0.187 ms): REAL_BULK planes by bulk copies (else a.bulk decides), REAL_SRC a
+// 256^3, 0.232 against 0.187 ms): REAL_BULK planes by bulk copies (XP = 0: a.bulk decides), REAL_SRC a
 // correction source (else none), REAL_EIGEN an eigenstress (else none).  BATCH: grid.z items, every workspace pointer
 // moved per item; a single solve's launch uses the arguments as they come.
 //
@@ -287,7 +312,7 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
   const int zc = min(a.zc, n3 - z0);
   const size_t rplane = (size_t)n2 * n1, rcomp = (size_t)n3 * rplane;
   constexpr bool has_src = FORCE && (OPT & REAL_SRC) != 0;
-  const bool bulk = (OPT & REAL_BULK) != 0 || a.bulk != 0;
+  const bool bulk = (OPT & REAL_BULK) != 0 || (XP == 0 && a.bulk != 0);
 
   const RealLayout lay = real_layout(xp, nthr, TY, has_src, (int)sizeof(T));
   const T* const ring = reinterpret_cast<const T*>(smraw + lay.ring);
