@@ -18,7 +18,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhs.so")
 UNITS = ["capi.cu", "kernels_util.cu", "noalloc.cu"] + [
     f"kernels_{part}_{prec}.cu" for prec in ("f64", "f32") for part in ("cols", "rows", "colp", "ext", "real_iso", "real_aniso")
-] + ["kernels_f32.cu", "kernels_f64.cu"]
+] + ["kernels_more_a_f32.cu", "kernels_more_b_f32.cu", "kernels_more_c_f32.cu", "kernels_f32.cu", "kernels_f64.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

@@ -1394,8 +1394,8 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
   };
   // compile-time plans: the default tile in the plan's block
   auto col_fixed = [&](int L, int* nthr) {
-    const int nt = hs::col_block(hs::fft_threads<hs::ColPlan>(L), 3 * c->ct, c->f64);
-    const bool fixed = hs::fft_fixed_length(L) && c->ct == (c->f64 ? 4 : 8) && (o.col_threads == 0 || o.col_threads == nt);
+    const int nt = hs::col_block(hs::fft_threads<hs::ColPlan>(L, c->f64), 3 * c->ct, c->f64);
+    const bool fixed = hs::fft_fixed_length(L, c->f64) && c->ct == (c->f64 ? 4 : 8) && (o.col_threads == 0 || o.col_threads == nt);
     *nthr = fixed ? nt : col_threads(L);
     return fixed;
   };
@@ -1482,7 +1482,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
   // persistent row passes: as many blocks as stay resident, at most one per batch
   {
     e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const size_t G = (size_t)(c->nthr_row / hs::fft_threads<hs::RowPlan>(c->n1));
+    const size_t G = (size_t)(c->nthr_row / hs::fft_threads<hs::RowPlan>(c->n1, c->f64));
     const size_t nbatch = ((size_t)3 * c->n2 * c->n3 / 2 + G - 1) / G;
     for (int m = 0; m < 2 && e == cudaSuccess; ++m) {
       int per_sm = 0;

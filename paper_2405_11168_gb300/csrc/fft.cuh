@@ -160,6 +160,13 @@ template <bool INV, typename C> struct Dft<12, INV, C> {
   static __device__ __forceinline__ void run(C* v) { dft_coprime<3, 4, 1, 3, INV>(v); }
 };
 
+template <bool INV, typename C> struct Dft<10, INV, C> {
+  static __device__ __forceinline__ void run(C* v) { dft_coprime<2, 5, 1, 3, INV>(v); }
+};
+template <bool INV, typename C> struct Dft<14, INV, C> {
+  static __device__ __forceinline__ void run(C* v) { dft_coprime<2, 7, 1, 4, INV>(v); }
+};
+
 // cos and sin of 2 pi j / P, 1 <= j <= (P - 1) / 2, for the odd prime radices
 template <int P> __host__ __device__ constexpr double prime_cos(int j) {
   if (P == 5) return j == 1 ? 0.30901699437494745 : -0.8090169943749473;
@@ -225,6 +232,39 @@ template <bool INV, typename C> struct Dft<8, INV, C> {
 template <bool INV, typename C> struct Dft<16, INV, C> {
   static __device__ __forceinline__ void run(C* v) { dft_composite<4, 4, INV>(v); }
 };
+
+// Two-float reals (h + l unevaluated, |l| below an ulp of h) for the butterflies of inverse FP32
+// transforms whose compile-time plan has a radix-11 stage.  A value there is rounded some nine times at
+// full size, and the strain is a difference of the transformed displacement, so that noise is what the FP32
+// iteration settles at (44^3: 1.25e-7 of the displacement per evaluation, 5e-6 of the stress in the
+// stiff phase).  With the inside of a butterfly in two floats a stage rounds once: 6e-8.
+struct df {
+  float h, l;
+  __device__ __forceinline__ df() {}
+  __device__ __forceinline__ constexpr df(double c) : h((float)c), l((float)(c - (double)(float)c)) {}
+  __device__ __forceinline__ constexpr df(float h_, float l_) : h(h_), l(l_) {}
+};
+__device__ __forceinline__ df operator+(df a, df b) {  // the sum of the high parts exactly (Knuth)
+  const float s = __fadd_rn(a.h, b.h), z = __fadd_rn(s, -a.h);
+  const float e = __fadd_rn(__fadd_rn(a.h, -__fadd_rn(s, -z)), __fadd_rn(b.h, -z));
+  return df(s, __fadd_rn(__fadd_rn(a.l, b.l), e));
+}
+__device__ __forceinline__ df operator-(df a) { return df(-a.h, -a.l); }
+__device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
+__device__ __forceinline__ df operator*(df a, df b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return df(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p))));
+}
+struct cdf {
+  df x, y;
+};
+__device__ __forceinline__ cdf widen(float2 a) {
+  cdf r;
+  r.x = df(a.x, 0.f);
+  r.y = df(a.y, 0.f);
+  return r;
+}
+__device__ __forceinline__ float2 narrow(cdf a) { return make_float2(a.x.h + a.x.l, a.y.h + a.y.l); }
 
 // 16-byte asynchronous global -> shared copies (cp.async, bypassing L1).
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
@@ -372,8 +412,9 @@ __host__ __device__ inline bool plan_ext(const FftPlan& p) {
 // ---------------------------------------------------------------------------
 // Compile-time plans: every stride, stage count and radix is a constant, so
 // the per-element index arithmetic folds away.  A plan is its radices and the
-// number of threads T that share a sequence, which divides L / r for every
-// radix r, so that no thread idles in any stage; a thread holds L / T values.
+// number of threads T that share a sequence; T divides L / r for every radix r
+// where it can, so that no thread idles in any stage.  A thread holds about
+// L / T values.
 // Few stages of large radices: a stage costs a load and a store of every value
 // through shared memory and two barriers.  Measured per pass (us, FP32, cubes): columns 128 as 8 x 16 15.5 y
 // and 27.5 z (8 x 4 x 4: 18.8, 38.7), 192 as 8 x 4 x 6 with 8 threads 35, 91 (4 x 4 x 12 with 16: 47, 110;
@@ -381,12 +422,14 @@ __host__ __device__ inline bool plan_ext(const FftPlan& p) {
 // 78, 188 (16 x 16: 78, 217); rows 256 as 16 x 16 81 and 73 (8 x 8 x 4: 87, 78), 192 as 4 x 4 x 12 48
 // (8 x 4 x 6: 67; run-time plan 84), 96 as 4 x 4 x 6 10.5 (8 x 12: 11.8), 128 in FP64 as 8 x 4 x 4 158 (8 x 16: 179).
 // ---------------------------------------------------------------------------
+// Lengths with a factor 5, 7 or 11 (FP32): as the run-time plan, whose index arithmetic, predicates and radix
+// switch cost three times the butterflies, a y pass of 112 took 38 us, a z pass of 88 58 and an x pass of
+// 160 37 (160 x 112 x 88).
 template <int LEN, int THREADS, int NST, int R0, int R1, int R2 = 1, int R3 = 1> struct FixedPlan {
   static constexpr int L = LEN, n = NST, T = THREADS;
   __host__ __device__ static constexpr int r(int i) { return i == 0 ? R0 : i == 1 ? R1 : i == 2 ? R2 : R3; }
   static_assert(R0 * R1 * R2 * R3 == L, "radices");
-  static_assert((L / R0) % T == 0 && (L / R1) % T == 0 && (NST < 3 || (L / R2) % T == 0) && (NST < 4 || (L / R3) % T == 0),
-                "threads");
+  static constexpr bool two_float = R0 == 11 || R1 == 11 || R2 == 11;  // see df
 };
 template <int L> struct ColPlan;
 template <> struct ColPlan<32> : FixedPlan<32, 4, 2, 4, 8> {};
@@ -398,31 +441,56 @@ template <> struct ColPlan<192> : FixedPlan<192, 8, 3, 8, 4, 6> {};
 template <> struct ColPlan<256> : FixedPlan<256, 32, 3, 8, 8, 4> {};
 template <> struct ColPlan<384> : FixedPlan<384, 32, 4, 4, 4, 4, 6> {};
 template <> struct ColPlan<512> : FixedPlan<512, 64, 3, 8, 8, 8> {};
+template <> struct ColPlan<40> : FixedPlan<40, 8, 2, 8, 5> {};
+template <> struct ColPlan<44> : FixedPlan<44, 4, 2, 4, 11> {};
+template <> struct ColPlan<56> : FixedPlan<56, 8, 2, 8, 7> {};
+template <> struct ColPlan<72> : FixedPlan<72, 6, 2, 12, 6> {};
+template <> struct ColPlan<80> : FixedPlan<80, 8, 2, 8, 10> {};
+template <> struct ColPlan<88> : FixedPlan<88, 8, 2, 8, 11> {};
+template <> struct ColPlan<112> : FixedPlan<112, 8, 2, 8, 14> {};
+template <> struct ColPlan<120> : FixedPlan<120, 12, 2, 12, 10> {};
+template <> struct ColPlan<144> : FixedPlan<144, 12, 2, 12, 12> {};
+template <> struct ColPlan<160> : FixedPlan<160, 10, 2, 16, 10> {};
+template <> struct ColPlan<176> : FixedPlan<176, 16, 2, 16, 11> {};
+template <> struct ColPlan<224> : FixedPlan<224, 16, 2, 16, 14> {};
+template <> struct ColPlan<240> : FixedPlan<240, 24, 3, 4, 6, 10> {};
+// rows: T a power of two that divides L
 template <int L> struct RowPlan : ColPlan<L> {};
+template <> struct RowPlan<72> : FixedPlan<72, 8, 2, 12, 6> {};
+template <> struct RowPlan<120> : FixedPlan<120, 8, 2, 12, 10> {};
+template <> struct RowPlan<144> : FixedPlan<144, 16, 2, 12, 12> {};
+template <> struct RowPlan<160> : FixedPlan<160, 16, 2, 16, 10> {};
+template <> struct RowPlan<240> : FixedPlan<240, 16, 3, 4, 6, 10> {};
 template <> struct RowPlan<96> : FixedPlan<96, 8, 3, 4, 4, 6> {};
 template <> struct RowPlan<128> : FixedPlan<128, 16, 3, 8, 4, 4> {};
 template <> struct RowPlan<192> : FixedPlan<192, 16, 3, 4, 4, 12> {};
 template <> struct RowPlan<256> : FixedPlan<256, 16, 2, 16, 16> {};
 #define HS_FIXED_LENGTHS(F) F(32) F(48) F(64) F(96) F(128) F(192) F(256) F(384) F(512)
+// FP32 only (FP64 runs their run-time plans: its passes wait for the FP64 pipe, not for the index arithmetic)
+#define HS_FIXED_LENGTHS_F32(F) \
+  F(40) F(44) F(56) F(72) F(80) F(88) F(112) F(120) F(144) F(160) F(176) F(224) F(240)
 
 // lengths whose column passes also run persistent
 #define HS_PERSISTENT_LENGTHS(F) F(128) F(192) F(256) F(384) F(512)
 
 // threads per sequence: the plan's, or one per kE values for the run-time plans
-template <template <int> class PLAN> __host__ __device__ inline int fft_threads(int L) {
+template <template <int> class PLAN> __host__ __device__ inline int fft_threads(int L, bool f64) {
   switch (L) {
 #define HS_CASE(LEN) case LEN: return PLAN<LEN>::T;
     HS_FIXED_LENGTHS(HS_CASE)
 #undef HS_CASE
-    default: return (L + kE - 1) / kE;
+#define HS_CASE(LEN) case LEN: if (!f64) return PLAN<LEN>::T; break;
+    HS_FIXED_LENGTHS_F32(HS_CASE)
+#undef HS_CASE
   }
+  return (L + kE - 1) / kE;
 }
-__host__ __device__ inline bool fft_fixed_length(int L) {
+__host__ __device__ inline bool fft_fixed_length(int L, bool f64) {
   switch (L) {
 #define HS_CASE(LEN) case LEN:
-    HS_FIXED_LENGTHS(HS_CASE)
+    HS_FIXED_LENGTHS(HS_CASE) return true;
+    HS_FIXED_LENGTHS_F32(HS_CASE) return !f64;
 #undef HS_CASE
-    return true;
     default: return false;
   }
 }
@@ -432,9 +500,13 @@ __host__ __device__ constexpr int ilog2_c(int v) { return v <= 1 ? 0 : 1 + ilog2
 // values a thread of the plan holds; above 8 the passes ask for fewer resident threads, so that the
 // values, a butterfly's temporaries and its twiddles stay in registers
 template <class PL> __host__ __device__ constexpr bool fft_wide() { return PL::L > 8 * PL::T; }
-// more than 16 values, or radix 12
+// more than 16 values, radix 12, or a long plan with radix 10 to 14 (us y, z with the tighter bound and its
+// spills -> this one: 176 40, 166 -> 36, 155; 224 80, 160 -> 63, 147; but 112 12.3, 22 -> 12.6, 26 and
+// the z pass of 88 41 -> 47, where the resident threads count for more)
 template <class PL> __host__ __device__ constexpr bool fft_very_wide() {
-  return PL::L > 16 * PL::T || PL::r(0) == 12 || PL::r(1) == 12 || PL::r(2) == 12 || PL::r(3) == 12;
+  for (int i = 0; i < 4; ++i)
+    if (PL::r(i) == 12 || (PL::L > 160 && PL::r(i) >= 10 && PL::r(i) <= 14)) return true;
+  return PL::L > 16 * PL::T;
 }
 
 // Block of a column pass over tiles of W sequences: the most sequences at a time that divide W (no thread
@@ -454,6 +526,7 @@ __host__ __device__ constexpr int col_block(int T, int W, bool f64) {
 template <int L> struct RowPos {
   static constexpr bool pow2 = (L & (L - 1)) == 0;
   static constexpr int T = RowPlan<L>::T;
+  static_assert((T & (T - 1)) == 0 && L % T == 0, "row positions");
   static constexpr int padded = L + L / T;
   static constexpr int pitch = L == 32 ? 36 : L == 64 ? 72 : pow2 ? L
                                : padded + (T >= 16 ? 0 : ((T - padded) % 16 + 16) % 16);
@@ -462,13 +535,16 @@ template <int L> struct RowPos {
          : pow2 ? e ^ (((e >> 2) ^ (e >> 3)) & 15) : e + (e >> ilog2_c(T));
   }
 };
-__host__ __device__ inline int row_pitch(int L) {
+__host__ __device__ inline int row_pitch(int L, bool f64) {
   switch (L) {
 #define HS_CASE(LEN) case LEN: return RowPos<LEN>::pitch;
     HS_FIXED_LENGTHS(HS_CASE)
 #undef HS_CASE
-    default: return rpitch(L);
+#define HS_CASE(LEN) case LEN: if (!f64) return RowPos<LEN>::pitch; break;
+    HS_FIXED_LENGTHS_F32(HS_CASE)
+#undef HS_CASE
   }
+  return rpitch(L);
 }
 // The swizzles are linear over XOR (shifts, XOR and masks are), and an index that is a sum of parts with
 // disjoint bits is their XOR, so at(a + b) = at(a) ^ at(b) for such parts; the padded positions are
@@ -520,13 +596,47 @@ template <bool TWS, typename C> __device__ __forceinline__ C tw_load(const C* __
   }
 }
 
+// Twiddles and DFT of one butterfly; output m to put(m, value).
+template <class PL, int R, int NS, bool INV, bool TWS, typename C, class Put>
+__device__ __forceinline__ void butterfly(C (&v)[R], const C* __restrict__ tw, int kk, int step, const Put& put) {
+  if constexpr (PL::two_float && INV && sizeof(C) == 8) {
+    cdf d[R];
+    d[0] = widen(v[0]);
+#pragma unroll
+    for (int m = 1; m < R; ++m) {
+      d[m] = widen(v[m]);
+      if (NS > 1) {
+        C w = stage_tw<TWS, PL, NS>(tw, m, kk, step);
+        w.y = -w.y;
+        d[m] = cmul(d[m], widen(w));
+      }
+    }
+    Dft<R, INV, cdf>::run(d);
+#pragma unroll
+    for (int m = 0; m < R; ++m) put(m, narrow(d[m]));
+  } else {
+    if (NS > 1) {
+#pragma unroll
+      for (int m = 1; m < R; ++m) {
+        C w = stage_tw<TWS, PL, NS>(tw, m, kk, step);
+        if (INV) w.y = -w.y;
+        v[m] = cmul(v[m], w);
+      }
+    }
+    Dft<R, INV, C>::run(v);
+#pragma unroll
+    for (int m = 0; m < R; ++m) put(m, v[m]);
+  }
+}
+
 // one stage on rows; element e of sequence s at buf[s * pitch + at(e)]
 template <class PL, int R, int NS, bool INV, bool TWS = false, typename C>
 __device__ __forceinline__ void stage_fixed(C* buf, int s, int t, bool active, const C* __restrict__ tw, bool wsync) {
   constexpr int L = PL::L, T = PL::T;
   using P = RowPos<L>;
   constexpr int nb = L / R;
-  constexpr int KB = nb / T;
+  constexpr int KB = (nb + T - 1) / T;
+  constexpr bool EXACT = nb % T == 0;
   constexpr int step = L / (NS * R);
   // power-of-two lengths: the stores' pq NS R + kk + m NS splits into disjoint parts too
   const int tin = P::at(t);
@@ -536,33 +646,23 @@ __device__ __forceinline__ void stage_fixed(C* buf, int s, int t, bool active, c
   if (active) {
 #pragma unroll
     for (int k = 0; k < KB; ++k)
+      if (EXACT || t + k * T < nb) {
 #pragma unroll
-      for (int m = 0; m < R; ++m) v[k][m] = sb[row_join<L>(tin, P::at(k * T + m * nb))];
+        for (int m = 0; m < R; ++m)
+          v[k][m] = sb[EXACT ? row_join<L>(tin, P::at(k * T + m * nb)) : P::at(t + k * T + m * nb)];
+      }
   }
   if (wsync) __syncwarp(); else __syncthreads();
   if (active) {
 #pragma unroll
     for (int k = 0; k < KB; ++k) {
       const int b = t + k * T;
-      const int kk = b % NS;
-      if (NS > 1) {
-#pragma unroll
-        for (int m = 1; m < R; ++m) {
-          C w = stage_tw<TWS, PL, NS>(tw, m, kk, step);
-          if (INV) w.y = -w.y;
-          v[k][m] = cmul(v[k][m], w);
-        }
-      }
-      Dft<R, INV, C>::run(v[k]);
+      if (!EXACT && b >= nb) continue;
       const int base = stockham_out<NS, R>(b);
-#pragma unroll
-      for (int m = 0; m < R; ++m) {
-        if constexpr (P::pow2) {
-          sb[tout ^ P::at((k * T / NS) * (NS * R) + (k * T) % NS + m * NS)] = v[k][m];
-        } else {
-          sb[P::at(base + m * NS)] = v[k][m];
-        }
-      }
+      butterfly<PL, R, NS, INV, TWS>(v[k], tw, b % NS, step, [&](int m, C x) {
+        if constexpr (P::pow2) sb[tout ^ P::at((k * T / NS) * (NS * R) + (k * T) % NS + m * NS)] = x;
+        else sb[P::at(base + m * NS)] = x;
+      });
     }
   }
   if (wsync) __syncwarp(); else __syncthreads();
@@ -614,14 +714,15 @@ __device__ __forceinline__ void stage_col(C* sm, const ColIO<C>& io, int s, int 
                                           const C* __restrict__ tw) {
   constexpr int L = PL::L, T = PL::T;
   constexpr int nb = L / R;
-  constexpr int KB = nb / T;
+  constexpr int KB = (nb + T - 1) / T;
+  constexpr bool EXACT = nb % T == 0;
   constexpr int step = L / (NS * R);
   const int c = s / CT, col = s - c * CT;
   C v[KB][R];
 #pragma unroll
   for (int k = 0; k < KB; ++k) {
     const int b = t + k * T;
-    if (active) {
+    if (active && (EXACT || b < nb)) {
       if (FROM_G) {
         const C* gp = io.gin + c * io.cstride + col;
         const bool ok = col < io.ccols;
@@ -637,31 +738,16 @@ __device__ __forceinline__ void stage_col(C* sm, const ColIO<C>& io, int s, int 
     }
   }
   if (!FROM_G) __syncthreads();
+  C* const gp = TO_G ? io.gout + c * io.cstride + col : nullptr;
 #pragma unroll
   for (int k = 0; k < KB; ++k) {
     const int b = t + k * T;
-    if (active) {
-      const int kk = b % NS;
-      if (NS > 1) {
-#pragma unroll
-        for (int m = 1; m < R; ++m) {
-          C w = stage_tw<TWS, PL, NS>(tw, m, kk, step);
-          if (INV) w.y = -w.y;
-          v[k][m] = cmul(v[k][m], w);
-        }
-      }
-      Dft<R, INV, C>::run(v[k]);
+    if (active && (EXACT || b < nb) && (!TO_G || col < io.ncol)) {
       const int base = stockham_out<NS, R>(b);
-      if (TO_G) {
-        if (col < io.ncol) {
-          C* gp = io.gout + c * io.cstride + col;
-#pragma unroll
-          for (int m = 0; m < R; ++m) gp[(size_t)(base + m * NS) * io.rstride] = v[k][m];
-        }
-      } else {
-#pragma unroll
-        for (int m = 0; m < R; ++m) sm[(base + m * NS) * W + s] = v[k][m];
-      }
+      butterfly<PL, R, NS, INV, TWS>(v[k], tw, b % NS, step, [&](int m, C x) {
+        if constexpr (TO_G) gp[(size_t)(base + m * NS) * io.rstride] = x;
+        else sm[(base + m * NS) * W + s] = x;
+      });
     }
   }
   if (!TO_G) __syncthreads();

@@ -60,6 +60,16 @@ template <typename T> static int col_length(const ColArgs<T>& a, int mode) {
   return (mode == COL_Y_FWD || mode == COL_Y_INV) ? a.n2 : a.n3;
 }
 
+// The FP32-only lengths (kernels_more_*_f32.cu); *ran: one of them with its block.
+template <int CT>
+static cudaError_t col_dispatch_f32(const ColArgs<float>& a, int mode, dim3 g, int nthr, size_t smem, cudaStream_t s,
+                                    bool* ran) {
+  const int L = col_length(a, mode);
+  *ran = fft_fixed_length(L, false) && nthr == col_block(fft_threads<ColPlan>(L, false), 3 * CT, false);
+  if (!*ran) return cudaSuccess;
+  return launch_col_more(a, mode, L, g, nthr, smem, s);
+}
+
 // compile-time variants for the default tile and block size at the lengths that have a plan
 template <typename T, int CT>
 static cudaError_t col_dispatch(const ColArgs<T>& a, int mode, dim3 g, int nthr, size_t smem, cudaStream_t s) {
@@ -73,6 +83,12 @@ static cudaError_t col_dispatch(const ColArgs<T>& a, int mode, dim3 g, int nthr,
     HS_FIXED_LENGTHS(HS_CASE)
 #undef HS_CASE
   }
+  if constexpr (sizeof(T) == 4) {
+    bool ran = false;
+    const cudaError_t e = col_dispatch_f32<CT>(a, mode, g, nthr, smem, s, &ran);
+    if (ran) return e;
+  }
+  if (plan_ext(a.plan)) return launch_col_ext<T>(a, mode, CT, g, nthr, smem, s);
   return col_ct<T, CT>(a, mode, g, nthr, smem, s);
 }
 
@@ -143,7 +159,9 @@ static cudaError_t row_occ(int n1, int nthr, size_t smem, int* n) {
       HS_FIXED_LENGTHS(HS_CASE)
 #undef HS_CASE
     }
+    if (sizeof(T) == 4 && fft_fixed_length(n1, false)) return launch_row_more(nullptr, MODE, n1, dim3(1), nthr, smem, nullptr, n);
   }
+  if (n1 % 5 == 0 || n1 % 7 == 0 || n1 % 11 == 0) return row_blocks_per_sm_ext<T>(MODE, nthr, smem, n);
   return row_occ_one<T, MODE>(nthr, smem, n);
 }
 template <typename T, int MODE>
@@ -154,7 +172,11 @@ static cudaError_t row_dispatch(const RowArgs<T>& a, dim3 nb, int nthr, size_t s
       HS_FIXED_LENGTHS(HS_CASE)
 #undef HS_CASE
     }
+    if constexpr (sizeof(T) == 4) {
+      if (fft_fixed_length(a.n1, false)) return launch_row_more(&a, MODE, a.n1, nb, nthr, smem, s, nullptr);
+    }
   }
+  if (plan_ext(a.plan)) return launch_row_ext<T>(a, MODE, nb, nthr, smem, s);
   return row_one<T, MODE>(a, nb, nthr, smem, s);
 }
 
@@ -228,8 +250,8 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
   cudaError_t launch_col<T>(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s) { \
     if (a.buf == nullptr || a.tw == nullptr || ((mode == COL_Z_GREEN || mode == COL_Z_INV_STATE) && a.S == nullptr)) \
       return cudaErrorInvalidValue; \
-    if (plan_ext(a.plan)) return launch_col_ext<T>(a, mode, ct, grid, nthr, smem, s); \
-    if (ct == (CT)) return col_ct<T, CT>(a, mode, grid, nthr, smem, s); \
+    if (ct == (CT)) return plan_ext(a.plan) ? launch_col_ext<T>(a, mode, ct, grid, nthr, smem, s) \
+                                            : col_ct<T, CT>(a, mode, grid, nthr, smem, s); \
     if (ct == (CT) / 2) return col_dispatch<T, (CT) / 2>(a, mode, grid, nthr, smem, s); \
     return cudaErrorInvalidValue; \
   } \
@@ -261,16 +283,23 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
     if (a.tw == nullptr || (mode == ROW_C2R ? (a.spec_in == nullptr || (a.real_out == nullptr && a.acc64 == nullptr)) \
                                             : (a.real_in == nullptr || a.spec_out == nullptr)))         \
       return cudaErrorInvalidValue;                                                                      \
-    if (plan_ext(a.plan)) return launch_row_ext<T>(a, mode, nb, nthr, smem, s);                        \
     return mode == ROW_C2R ? row_dispatch<T, ROW_C2R>(a, nb, nthr, smem, s)                             \
                            : row_dispatch<T, ROW_R2C>(a, nb, nthr, smem, s);                            \
   }                                                                                                      \
   template <>                                                                                            \
   cudaError_t row_blocks_per_sm<T>(int mode, int n1, int nthr, size_t smem, int* n) {                     \
-    if (n1 % 5 == 0 || n1 % 7 == 0 || n1 % 11 == 0) return row_blocks_per_sm_ext<T>(mode, nthr, smem, n);  \
     return mode == ROW_C2R ? row_occ<T, ROW_C2R>(n1, nthr, smem, n) : row_occ<T, ROW_R2C>(n1, nthr, smem, n); \
   }                                                                                                      \
   }
+
+// A group of the FP32-only lengths: column passes (cases of launch_col_more's switch) and row passes, whose
+// kernels serve single and batched launches.
+#define HS_COL_MORE_CASE(LEN)                                                                             \
+  case LEN: return col_ct<float, 8, LEN, col_block(ColPlan<LEN>::T, 24, false)>(a, mode, grid, nthr, smem, s);
+#define HS_ROW_MORE_CASE(LEN)                                                                             \
+  case LEN:                                                                                              \
+    if (occ != nullptr) return row_occ_one<float, MODE, LEN>(nthr, smem, occ);                            \
+    return row_launch<float, MODE, LEN, true>(*a, nb, nthr, smem, s);
 
 // Kernels for plans with a radix-5, 7 or 11 stage, in their own translation unit.
 #define HS_INSTANTIATE_EXT(T, CT)                                                                         \

@@ -72,6 +72,11 @@ cudaError_t colp_blocks_per_sm(int mode, int L, int ct, int nthr, size_t smem, i
 template <typename T>
 cudaError_t launch_row(const RowArgs<T>& a, int mode, dim3 grid, int nthr, size_t smem, cudaStream_t s);
 
+// column and row passes of the FP32-only compile-time lengths; a null: *occ = resident blocks per SM
+cudaError_t launch_col_more(const ColArgs<float>& a, int mode, int L, dim3 grid, int nthr, size_t smem, cudaStream_t s);
+cudaError_t launch_row_more(const RowArgs<float>* a, int mode, int L, dim3 grid, int nthr, size_t smem, cudaStream_t s,
+                            int* occ);
+
 // the same passes for plans with a radix-5, 7 or 11 stage (default column tile only)
 template <typename T>
 cudaError_t launch_col_ext(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s);

@@ -75,8 +75,8 @@ struct RowLayout {
 };
 __host__ __device__ inline RowLayout row_layout(int mode, int n1, int P, int nthr, int tsize) {
   RowLayout L;
-  L.G = nthr / fft_threads<RowPlan>(n1);
-  L.zbytes = (((size_t)L.G * row_pitch(n1) * 2 * tsize) + 15) & ~(size_t)15;
+  L.G = nthr / fft_threads<RowPlan>(n1, tsize == 8);
+  L.zbytes = (((size_t)L.G * row_pitch(n1, tsize == 8) * 2 * tsize) + 15) & ~(size_t)15;
   L.rowbytes = (mode == ROW_C2R) ? (size_t)P * 2 * tsize : (size_t)n1 * tsize;
   L.outbytes = (mode == ROW_C2R) ? (size_t)n1 * tsize : (size_t)P * 2 * tsize;
   const size_t rb = L.rowbytes > L.outbytes ? L.rowbytes : L.outbytes;
