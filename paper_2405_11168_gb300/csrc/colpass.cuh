@@ -313,7 +313,6 @@ __global__ void __launch_bounds__(col_max_threads(NT, sizeof(T) == 8), col_min_b
   using C = typename cplx_t<T>::type;
   static_assert(!TMA || (MODE != COL_Z_INV_STATE && LF > 0), "tensor copies: fixed lengths, iteration modes");
   const ColArgs<T> a = col_item_args(a_);
-  if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   extern __shared__ __align__(128) unsigned char smraw[];
   // TMA: the tile starts on a 128-byte boundary and its barrier follows it (kColpTmaSlack)
   unsigned char* const smb = TMA ? smraw + ((128u - (smem_u32(smraw) & 127u)) & 127u) : smraw;
@@ -351,6 +350,9 @@ __global__ void __launch_bounds__(col_max_threads(NT, sizeof(T) == 8), col_min_b
         for (int i = tid; i < L; i += nthr) tzs[i] = __ldg(tw + i);
     }
   };
+  copy_tables();
+  pass_wait();
+  if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   if constexpr (TMA) {
     uint64_t* const tbar = reinterpret_cast<uint64_t*>(smb + (size_t)L * W * sizeof(C));
     // the copy needs a 128-byte aligned destination and a 64-byte aligned map: checked once,
@@ -375,7 +377,6 @@ __global__ void __launch_bounds__(col_max_threads(NT, sizeof(T) == 8), col_min_b
         asm volatile("prefetch.global.L2 [%0];\n" ::"l"(a.S + c * cstride + base + e * rstride));
       }
     }
-    copy_tables();
     __syncthreads();  // the barrier is initialised before anyone waits on it
     if (!mbar_wait(tbar, 0)) {
       if (tid == 0) a.st->done = DONE_TIMEOUT;
@@ -418,7 +419,6 @@ __global__ void __launch_bounds__(col_max_threads(NT, sizeof(T) == 8), col_min_b
   } else {
     cp_async_wait_all();
   }
-  if (!TMA) copy_tables();
   __syncthreads();
   if constexpr (LF > 0) {
     // compile-time plan; the last stage writes straight to global memory
@@ -442,8 +442,10 @@ __global__ void __launch_bounds__(col_max_threads(NT, sizeof(T) == 8), col_min_b
         col_green<T, CT>(a, sm, ss, base, rstride, cstride, x0, outer, ncol, L, tid, nthr);
       }
       __syncthreads();
+      pass_begin();
       fft_col_fixed<ColPlan<LF>, W, CT, true, false, true, true>(sm, io, tws, tid, nthr);
     } else {
+      pass_begin();
       fft_col_fixed<ColPlan<LF>, W, CT, MODE == COL_Y_INV || MODE == COL_Z_INV_STATE, false, true, true>(sm, io, tws, tid,
                                                                                             nthr);
     }
@@ -483,7 +485,6 @@ __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<
   static_assert(LF > 0 && MODE != COL_Z_INV_STATE, "persistent column pass: fixed lengths, iteration modes");
   static_assert(!TMA || MODE == COL_Y_FWD || MODE == COL_Y_INV || MODE == COL_Z_GREEN, "tensor copies");
   const ColArgs<T> a = col_item_args(a_);
-  if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   extern __shared__ __align__(128) unsigned char smraw[];
   constexpr bool yaxis = (MODE == COL_Y_FWD || MODE == COL_Y_INV);
   constexpr int L = LF, W = 3 * CT;
@@ -499,6 +500,7 @@ __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<
     // the copy needs a 128-byte aligned destination and a 64-byte aligned map: checked once,
     // the pass ends with an error status instead of issuing a misaligned copy
     if ((smem_u32(sm0) & 127u) != 0 || (reinterpret_cast<uintptr_t>(&a_.tmap) & 63u) != 0) {
+      pass_wait();
       if (tid == 0) a.st->done = DONE_FAULT;
       return;
     }
@@ -552,6 +554,8 @@ __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<
   stage_twiddles<ColPlan<LF>>(tws, a.tw, tid, NT);
   if (MODE == COL_Z_GREEN)
     for (int i = tid; i < L; i += NT) tzs[i] = __ldg(a.tw + i);
+  pass_wait();
+  if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   bool timed_out = false;
   int t = blockIdx.x;
   if constexpr (TMA) {
@@ -589,6 +593,7 @@ __global__ void __launch_bounds__(NT, 2) k_colp(const __grid_constant__ ColArgs<
     io.rstride = rstride;
     io.ccols = min(CT, a.P - x0);
     io.ncol = min(CT, a.nh - x0);
+    if (t + (int)gridDim.x >= ntiles) pass_begin();
     if (MODE == COL_Z_GREEN) {
       fft_col_fixed<ColPlan<LF>, W, CT, false, false, false, true>(sm, io, tws, tid, NT);
       col_green_fixed<T, CT, LF, NT>(a, sm, base, rstride, cstride, x0, outer, io.ncol, tid, tzs);

@@ -42,6 +42,15 @@ struct DevStatus {
 // kernel's own check (the alignment a tensor copy needs) failed before the access.  Both stay set.
 enum { DONE_RUNNING = 0, DONE_CONVERGED = 1, DONE_MAXITER = 2, DONE_DIVERGED = 3, DONE_TIMEOUT = 4, DONE_FAULT = 5 };
 
+// Programmatic dependents: once every block of a pass has called pass_begin or ended, the next pass's blocks may start;
+// pass_wait holds them until this pass has finished and its writes are visible.  Every kernel
+// launched as a dependent calls pass_wait before it ends, so that finished means the whole chain before it,
+// and until then touches only what no kernel writes: its arguments, shared memory and the twiddle
+// tables.  Called early, pass_begin packs the next pass's blocks onto the SMs that are free first: 64^3 FP64
+// 277 -> 442 us per evaluation, 256^3 FP32 650 -> 689.  So a pass calls it before its last transform.
+__device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Batched launches (one launch over many solves of the same grid): item
 // blockIdx.z works in the workspace that starts zstride bytes after item
 // blockIdx.z - 1's, so every workspace pointer of the launch moves by

@@ -137,12 +137,29 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
     k_row(const RowArgs<T> a_) {
   using C = typename cplx_t<T>::type;
   const RowArgs<T> a = BATCH ? row_item_args(a_) : a_;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int tid = threadIdx.x, nthr = LF > 0 ? 256 : (int)blockDim.x;
+  const int n1 = LF > 0 ? LF : a.n1, P = a.P, nh = n1 / 2 + 1, half = n1 / 2;
+  const RowLayout L = row_layout(MODE, n1, P, nthr, (int)sizeof(T));
+  // fixed lengths: the transforms read their twiddles from the plan's per-stage table in shared
+  // memory, and each batch arrives by one bulk copy on its staging buffer's mbarrier (waits
+  // bounded; a timeout is recorded in the status)
+  C* const tws = reinterpret_cast<C*>(smraw + L.tws);
+  const bool bload = LF > 0 && (L.rowbytes & 15) == 0;
+  uint64_t* sbar = reinterpret_cast<uint64_t*>(smraw + L.bar);
+  if constexpr (LF > 0) stage_twiddles<RowPlan<LF>>(tws, a.tw, tid, nthr);
+  if (bload && tid == 0) {
+    mbar_init(sbar, 1);
+    mbar_init(sbar + 1, 1);
+    mbar_init_fence();
+  }
+  if (LF > 0) __syncthreads();
+  pass_wait();
   // In the pass that takes the stopping test the done flag may change while blocks start: the block
   // decides as one.
   bool skip = a.st->retired || (a.skip_if_done && a.st->done);
   if (MODE == ROW_R2C) skip = __syncthreads_or(skip);
   if (skip) return;
-  extern __shared__ __align__(16) unsigned char smraw[];
   // The stopping test of this evaluation runs beside the row transforms instead of at the end of the
   // real-space pass, where the whole chip waited for one block (12 of 31 us at 64^3).  A done flag
   // that it sets is seen by the next kernels; blocks of this one that see it early skip rows nobody reads.
@@ -152,9 +169,6 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
     return;
   }
   const int blk = (int)blockIdx.x - nfin, nblk = (int)gridDim.x - nfin;
-  const int n1 = LF > 0 ? LF : a.n1, P = a.P, nh = n1 / 2 + 1, half = n1 / 2;
-  const int tid = threadIdx.x, nthr = LF > 0 ? 256 : (int)blockDim.x;
-  const RowLayout L = row_layout(MODE, n1, P, nthr, (int)sizeof(T));
   const int T8 = LF > 0 ? RowPlan<(LF > 0 ? LF : 64)>::T : (n1 + kE - 1) / kE;  // threads per sequence
   const int G = L.G;                           // sequences per batch
   const int grp = tid / T8, t = tid - grp * T8;
@@ -182,23 +196,7 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
   // buffer and written by one bulk copy (FP64 accumulation keeps per-element
   // updates).  R2C measured faster with direct stores (0.104 vs 0.112 ms at 256^3).
   const bool bulk = LF > 0 && MODE == ROW_C2R && a.acc64 == nullptr && (L.outbytes & 15) == 0;
-  // fixed lengths: each batch arrives by one bulk copy on its staging buffer's mbarrier (waits
-  // bounded; a timeout is recorded in the status)
-  const bool bload = LF > 0 && (L.rowbytes & 15) == 0;
-  uint64_t* sbar = reinterpret_cast<uint64_t*>(smraw + L.bar);
   bool timed_out = false;
-  if (bload) {
-    if (tid == 0) {
-      mbar_init(sbar, 1);
-      mbar_init(sbar + 1, 1);
-      mbar_init_fence();
-    }
-    __syncthreads();
-  }
-  // fixed lengths: the transforms read their twiddles from the plan's per-stage table in shared
-  // memory (first read after the barrier that opens the first batch)
-  C* const tws = reinterpret_cast<C*>(smraw + L.tws);
-  if constexpr (LF > 0) stage_twiddles<RowPlan<LF>>(tws, a.tw, tid, nthr);
   int buf = 0;
   if (blk < nbatch && (!bload || tid == 0)) row_stage<T, MODE>(a, L, smraw, blk, 0, bload);
   int k = 0;
@@ -208,6 +206,7 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
     if (bulk && tid == 0) bulk_wait_read_all();  // staging buffer buf ^ 1 is free again
     __syncthreads();
     if (b + nblk < nbatch && (!bload || tid == 0)) row_stage<T, MODE>(a, L, smraw, b + nblk, buf ^ 1, bload);
+    if (b + nblk >= nbatch) pass_begin();
     unsigned char* stg = smraw + L.zbytes + (size_t)buf * L.stage;
     const size_t nr = min((size_t)2 * G, (size_t)a.nrows - 2 * (size_t)b * G);
     const int s = b * G + grp;
