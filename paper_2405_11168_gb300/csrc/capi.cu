@@ -503,7 +503,8 @@ int pick_ty(int n2) { return (n2 % 4 == 0) ? 4 : 2; }
 
 size_t march_smem(int n1, int ty, bool f64, int mode, bool real, bool has_src = false) {
   const int nthr = ((n1 + 31) / 32) * 32, ts = f64 ? 8 : 4;
-  if (real) return hs::real_layout(hs::real_pitch(f64, ty, mode, n1), nthr, ty, has_src, ts).total;
+  if (real)
+    return hs::real_layout(hs::real_pitch(f64, ty, mode, n1), hs::real_threads(f64, ty, n1), ty, has_src, ts).total;
   return hs::march_layout(n1, pitch_of(n1 / 2 + 1, f64), nthr, ty, mode, has_src, ts).total;
 }
 
@@ -685,7 +686,8 @@ template <typename T> hs_status launch_stencil(hs_ctx* c, const double E[6], con
   cudaError_t e;
   {
     LaunchScope ls(c, mode == hs::MODE_FORCE ? (src != nullptr ? HS_K_XPASS_SRC : HS_K_XPASS) : HS_K_FIELDS);
-    e = hs::launch_real<T>(a, c->iso, c->ty, mode, zg(c, c->grid_m), c->nthr_m, sm, c->stream);
+    e = hs::launch_real<T>(a, c->iso, c->ty, mode, zg(c, c->grid_m), hs::real_threads(c->f64, c->ty, c->n1), sm,
+                           c->stream);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "k_real");
   return HS_OK;
@@ -1002,7 +1004,8 @@ hs_status launch_residual64(hs_ctx* c, const double E[6], int mode, void* eps, v
   a.skip_if_done = 0;
   const size_t sm = march_smem(c->n1, c->ty64, true, mode, true);
   LaunchScope ls(c, mode == hs::MODE_FIELDS ? HS_K_FIELDS : HS_K_RESID64);
-  cudaError_t e = hs::launch_real<double>(a, c->iso, c->ty64, mode, zg(c, c->grid_m64), c->nthr_m, sm, c->stream);
+  cudaError_t e = hs::launch_real<double>(a, c->iso, c->ty64, mode, zg(c, c->grid_m64),
+                                          hs::real_threads(true, c->ty64, c->n1), sm, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "k_real(residual fp64)");
   return HS_OK;
 }
@@ -1434,9 +1437,11 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int nwarps = c->nthr_m / 32;
   auto real_smem = [&](int ty, bool f64, bool src) { return march_smem(c->n1, ty, f64, hs::MODE_FORCE, true, src); };
-  auto tile_fits = [&](int ty, bool f64) { return real_smem(ty, f64, !f64) <= (size_t)smem_optin; };
+  auto tile_fits = [&](int ty, bool f64) {
+    return hs::real_rows_fit(f64, ty, c->n1) && real_smem(ty, f64, !f64) <= (size_t)smem_optin;
+  };
   auto pick64 = [&](int fixed_ty, int fixed_zc, int* ty, int* zc) {
-    hs::pick_tile64(c->iso, c->n1, c->n2, c->n3, fixed_ty, (size_t)smem_optin, std::max(1, nsm), 0, ty, zc);
+    hs::pick_tile64(c->iso, c->n1, c->n2, c->n3, fixed_ty, (size_t)smem_optin, std::max(1, nsm), 0, true, ty, zc);
     if (fixed_zc > 0) *zc = std::min(fixed_zc, c->n3);
   };
   int ytile = o.ytile;
@@ -1455,7 +1460,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
       c->zc = o.zchunk > 0 ? std::min(o.zchunk, c->n3)
                            : hs::pick_zchunk32(c->n2 / c->ty, c->n3, nwarps, std::max(1, occ), std::max(1, nsm));
     }
-    c->grid_m = dim3(c->n2 / c->ty, (c->n3 + c->zc - 1) / c->zc);
+    c->grid_m = dim3(c->n2 / c->ty * hs::real_halves(c->f64, c->ty, c->n1), (c->n3 + c->zc - 1) / c->zc);
   }
   c->ty64 = c->ty;
   c->zc64 = c->zc;
@@ -1464,7 +1469,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
     while (t > 2 && !tile_fits(t, true)) t /= 2;
     pick64(t, 0, &c->ty64, &c->zc64);
   }
-  c->grid_m64 = dim3(c->n2 / c->ty64, (c->n3 + c->zc64 - 1) / c->zc64);
+  c->grid_m64 = dim3(c->n2 / c->ty64 * hs::real_halves(true, c->ty64, c->n1), (c->n3 + c->zc64 - 1) / c->zc64);
   // z pass: the state tile in shared memory beside the force tile when asked for (col_state = 2)
   if (o.col_state == 2 && 2 * c->smem_z <= (size_t)smem_optin) {
     c->zstate_smem = true;

@@ -12,8 +12,25 @@ static cudaError_t real_one(const MarchArgs<T>& a, dim3 g, int nthr, size_t smem
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   if (occ != nullptr) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, nthr, smem);
-  k<<<g, nthr, smem, s>>>(a, MAT{a.mat});
-  return cudaGetLastError();
+  if constexpr ((OPT & REAL_SPLIT) != 0) {
+    if (!a.bulk || nthr != real_threads(true, TY, a.n1)) return cudaErrorInvalidValue;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = dim3((unsigned)nthr);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, a, MAT{a.mat});
+  } else {
+    k<<<g, nthr, smem, s>>>(a, MAT{a.mat});
+    return cudaGetLastError();
+  }
 }
 
 // batched launches (zstride != 0) run the force pass without an eigenstrain only
@@ -45,6 +62,10 @@ static cudaError_t real_opt(const MarchArgs<T>& a, dim3 g, int nthr, size_t smem
 template <typename T, int TY, class MAT, int MODE>
 static cudaError_t real_xp(const MarchArgs<T>& a, dim3 g, int nthr, size_t smem, cudaStream_t s, int* occ) {
   if constexpr (sizeof(T) == 8) {
+    if constexpr (TY == 8) {
+      if (!real_rows_fit(true, TY, a.n1)) return cudaErrorInvalidValue;
+      if (real_split(true, TY, a.n1)) return real_opt<T, TY, MAT, MODE, 0, 256, REAL_SPLIT>(a, g, nthr, smem, s, occ);
+    }
     if (nthr <= 256) return real_opt<T, TY, MAT, MODE, 0, 256>(a, g, nthr, smem, s, occ);
     if constexpr (TY < 8) return real_opt<T, TY, MAT, MODE, 0, 512>(a, g, nthr, smem, s, occ);
     else return cudaErrorInvalidValue;

@@ -35,14 +35,20 @@ inline int real_pitch_class(bool f64, int ty, int mode, int n1) {
   if (f64 || ty != 4 || mode != MODE_FORCE) return 0;
   return n1 <= 64 ? 64 : n1 <= 128 ? 128 : n1 <= 256 ? 256 : 512;
 }
+// FP64 tiles of 8 rows of more than 256 columns: two blocks of a cluster take half the columns each
+// (N1 a multiple of 16, so that bulk copies take half rows).  The columns and threads of a block.
+inline bool real_split(bool f64, int ty, int n1) { return f64 && ty == 8 && n1 > 256; }
+inline bool real_rows_fit(bool f64, int ty, int n1) { return !real_split(f64, ty, n1) || n1 % 16 == 0; }
+inline int real_halves(bool f64, int ty, int n1) { return real_split(f64, ty, n1) ? 2 : 1; }
+inline int real_threads(bool f64, int ty, int n1) { return (n1 / real_halves(f64, ty, n1) + 31) / 32 * 32; }
 // Its row pitch in shared memory.
 inline int real_pitch(bool f64, int ty, int mode, int n1) {
   const int c = real_pitch_class(f64, ty, mode, n1);
-  return c > 0 ? c : (n1 + 7) & ~7;
+  return c > 0 ? c : real_split(f64, ty, n1) ? n1 / 2 + 8 : (n1 + 7) & ~7;
 }
 
 // The pass on a real displacement field (k_real): mode MODE_FORCE / MODE_FIELDS / MODE_FORCE_FIELDS (FP64
-// only); a.xp as real_pitch() gives it.  occ: not null: the resident blocks per SM instead of a launch.
+// only); grid: (N2 / ty * real_halves(), z chunks, items), real_threads() threads; a.xp as real_pitch() gives it.  occ: not null: the resident blocks per SM instead of a launch.
 template <typename T, bool ISO>
 cudaError_t launch_real_law(const MarchArgs<T>& a, int ty, int mode, dim3 grid, int nthr, size_t smem, cudaStream_t s,
                             int* occ);

@@ -37,7 +37,8 @@ template <typename K> static cudaError_t set_smem(K kernel, size_t smem) {
   return e;
 }
 
-// Launch of a transform pass.  FP32 passes of a solve over at most 2^22 voxels launch as programmatic dependents of the kernel before them: their blocks start and fill their twiddle tables while that kernel's
+// Launch of a transform pass.  FP32 passes of a solve over at most 2^22 voxels launch as programmatic
+// dependents of the kernel before them: their blocks start and fill their twiddle tables while that kernel's
 // last transforms run (pass_begin), and wait for its results in pass_wait.  us per evaluation: 64^3 37.2 ->
 // 34.5, 96^3 60.7 -> 58.5, 128^3 101.4 -> 97.5, but 192^3 328 -> 326 and 256^3 651 -> 655; in FP64, whose passes
 // need their blocks spread evenly over the SMs, 64^3 277 -> 326 and 128^3 1749 -> 1894.  The real-space pass

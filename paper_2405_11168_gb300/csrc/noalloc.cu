@@ -97,7 +97,6 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
   for (int i = 0; i < 6; ++i)
     if (!std::isfinite(E[i])) return HS_ERR_INVALID_ARG;
   const int n1 = grid[0], n2 = grid[1], n3 = grid[2];
-  const int nthr = ((n1 + 31) / 32) * 32;
   int dev = 0, smem_optin = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
@@ -125,11 +124,13 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
   }
 
   // rows per block and z chunk: as the FP64 sweeps of hs_solve, within the partial sums the array holds
+  // (rows of more than 256 columns in halves need bulk copies)
   int ty = 2, zc = 1;
-  hs::pick_tile64(iso, n1, n2, n3, 0, (size_t)smem_optin, std::max(1, nsm), HS_NOALLOC_MAX_BLOCKS, &ty, &zc);
+  const bool bulk = n1 % 8 == 0 && reinterpret_cast<uintptr_t>(u) % 16 == 0 && reinterpret_cast<uintptr_t>(ids) % 16 == 0;
+  hs::pick_tile64(iso, n1, n2, n3, 0, (size_t)smem_optin, std::max(1, nsm), HS_NOALLOC_MAX_BLOCKS, bulk, &ty, &zc);
   const size_t smem = hs::real_bytes(true, n1, ty, false);
   if (smem > (size_t)smem_optin) return HS_ERR_UNSUPPORTED_SIZE;
-  const int ytiles = n2 / ty, nzc = (n3 + zc - 1) / zc;
+  const int ytiles = n2 / ty * hs::real_halves(true, ty, n1), nzc = (n3 + zc - 1) / zc;
   if ((size_t)ytiles * nzc > (size_t)HS_NOALLOC_MAX_BLOCKS) return HS_ERR_UNSUPPORTED_SIZE;
 
   unsigned char* base = nullptr;
@@ -187,8 +188,8 @@ extern "C" hs_status hs_residual_noalloc(const int grid[3], const unsigned short
   a.skip_if_done = 0;
   a.xp = hs::real_pitch(true, ty, hs::MODE_FORCE, n1);
   // bulk copies need rows that start and end on 16 bytes; the caller's pointers may not
-  a.bulk = (n1 % 8 == 0 && reinterpret_cast<uintptr_t>(u) % 16 == 0 && reinterpret_cast<uintptr_t>(ids) % 16 == 0) ? 1 : 0;
-  e = hs::launch_real<double>(a, iso, ty, hs::MODE_FORCE, dim3(ytiles, nzc), nthr, smem, s);
+  a.bulk = bulk ? 1 : 0;
+  e = hs::launch_real<double>(a, iso, ty, hs::MODE_FORCE, dim3(ytiles, nzc), hs::real_threads(true, ty, n1), smem, s);
   if (e != cudaSuccess) return HS_ERR_CUDA;
   e = cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -28,7 +28,7 @@
 
 namespace hs {
 
-enum { REAL_BULK = 1, REAL_SRC = 2, REAL_EIGEN = 4 };
+enum { REAL_BULK = 1, REAL_SRC = 2, REAL_EIGEN = 4, REAL_SPLIT = 8 };
 
 template <typename T> struct Pair;  // two-lane arithmetic, every operation rounded lane by lane
 template <> struct Pair<float> {
@@ -217,6 +217,65 @@ __device__ __forceinline__ void real_prefetch_bulk(const MarchArgs<T>& a, const 
   }
 }
 
+// The same for half a row (REAL_SPLIT): columns x0 .. x0 + nx - 1 from position 2 of a ring row on, the two columns
+// on their left before them (periodic), ids of the block's columns.  x0 is 0 or a multiple of 8.
+template <typename T, int TY>
+__device__ __forceinline__ void real_prefetch_half(const MarchArgs<T>& a, const RealLayout& lay, unsigned char* sm,
+                                                   int xp, int x0, int nx, int y0, int pu, int slot, int ib, uint64_t* bar) {
+  constexpr int NR = TY + 2;
+  const int n1 = a.n1, n2 = a.n2, n3 = a.n3, lane = threadIdx.x & 31;
+  const size_t rplane = (size_t)n2 * n1, rcomp = (size_t)n3 * rplane;
+  const int gz = pu < 0 ? pu + n3 : (pu >= n3 ? pu - n3 : pu);
+  const int nu = 3 * NR, ni = ib >= 0 ? TY + 1 : 0;
+  if (lane == 0) mbar_arrive_expect_tx(bar, (unsigned)(nu * (nx + 2) * sizeof(T) + ni * nx * 2));
+  __syncwarp();
+  auto copy = [&](void* dst, const void* src, unsigned bytes) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+  };
+  T* const ru = reinterpret_cast<T*>(sm + lay.ring) + (size_t)slot * nu * xp;
+  uint16_t* const ri = reinterpret_cast<uint16_t*>(sm + lay.ids) + (size_t)ib * (TY + 1) * xp;
+  for (int i = lane; i < nu + ni; i += 32) {
+    if (i < nu) {
+      const int c = i / NR, gy = (y0 - 1 + (i - c * NR) + n2) % n2;
+      const T* const row = a.ureal + c * rcomp + (size_t)gz * rplane + (size_t)gy * n1;
+      T* const d = ru + (size_t)i * xp;
+      if (x0 > 0) {
+        copy(d, row + x0 - 2, (unsigned)((nx + 2) * sizeof(T)));
+      } else {
+        copy(d, row + n1 - 2, (unsigned)(2 * sizeof(T)));
+        copy(d + 2, row, (unsigned)(nx * sizeof(T)));
+      }
+    } else {
+      const int r = i - nu, gy = (y0 + r) % n2;
+      copy(ri + (size_t)r * xp, a.ids + (size_t)gz * rplane + (size_t)gy * n1 + x0, (unsigned)(nx * 2));
+    }
+  }
+}
+
+// Barrier of the two blocks of a cluster, with the shared-memory writes before it visible to both after it; a
+// word of the other block's shared memory.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ unsigned peer_addr(const void* p, int peer) {
+  unsigned a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(peer));
+  return a;
+}
+__device__ __forceinline__ double peer_load(const double* p, int peer) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(v) : "r"(peer_addr(p, peer)) : "memory");
+  return v;
+}
+__device__ __forceinline__ int peer_load(const int* p, int peer) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(v) : "r"(peer_addr(p, peer)) : "memory");
+  return v;
+}
+
 // Rows of n elements of E bytes by the block's warps, one row per warp and turn: cp.async in the widest chunks
 // (16, 8 or 4 bytes) that start and end every row; 2-byte rows that do not start on 4 bytes element by element.
 // Every thread over every row in turn, 8 bytes at a time, left most of a block without a copy; rows per warp and the
@@ -291,28 +350,40 @@ __device__ __forceinline__ void real_prefetch_async(const MarchArgs<T>& a, const
 // A step handles voxel plane p between corner planes p - 1 and p (ring slots filled two steps ahead)
 // and completes corner plane p - 1.  One block barrier per step: it publishes the left-going sums of
 // each warp's first column, which the previous warp's last column needs, and frees ring slot p - 2.
+//
+// REAL_SPLIT (FP64, more than 256 columns): the two blocks of a cluster take half the columns each, the barrier
+// of a step is the cluster's, and a half's last column reads the sums of the other half's first one from
+// that block's shared memory.  One block of 512 threads has 128 registers and shared memory for tiles of 2
+// rows, which compute 3 voxel rows for 2; halves of 256 run 8 rows with 255 registers: FP64 sweep of 512^3, 21-constant
+// law, 64.1 -> 51.6 ms.
 template <typename T, int TY, class MAT, int MODE, int XP, int NT, int OPT, bool BATCH>
 __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT mat_) {
   using P = Pair<T>;
   using V = typename P::V;
   constexpr int NR = TY + 2;
   constexpr bool F64 = sizeof(T) == 8;
+  constexpr bool SPLIT = (OPT & REAL_SPLIT) != 0;
   constexpr bool FORCE = MODE == MODE_FORCE || MODE == MODE_FORCE_FIELDS;
   constexpr bool FIELDS = MODE == MODE_FIELDS || MODE == MODE_FORCE_FIELDS;
   const MarchArgs<T> a = BATCH ? march_item_args(a_) : a_;
   MAT mat = mat_;
   if (BATCH) mat.tab = a.mat;
-  if (a.st->retired || (a.skip_if_done && a.st->done)) return;
+  bool skip = false;
+  if constexpr (SPLIT) skip = a.st->retired || (a.skip_if_done && a.st->done);
+  else if (a.st->retired || (a.skip_if_done && a.st->done)) return;
   extern __shared__ __align__(128) unsigned char smraw[];
   const int n1 = a.n1, n2 = a.n2, n3 = a.n3;
   const int xp = XP > 0 ? XP : a.xp;
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
-  const int y0 = blockIdx.x * TY;
+  constexpr int XO = SPLIT ? 2 : 0;  // position of the block's first column in a ring row
+  const int half = SPLIT ? (int)(blockIdx.x & 1) : 0;  // also the rank in the cluster
+  const int nx = SPLIT ? n1 >> 1 : n1, x0 = SPLIT ? half * nx : 0;  // columns of the block
+  const int y0 = (SPLIT ? blockIdx.x >> 1 : blockIdx.x) * TY;
   const int z0 = blockIdx.y * a.zc;
   const int zc = min(a.zc, n3 - z0);
   const size_t rplane = (size_t)n2 * n1, rcomp = (size_t)n3 * rplane;
   constexpr bool has_src = FORCE && (OPT & REAL_SRC) != 0;
-  const bool bulk = (OPT & REAL_BULK) != 0 || (XP == 0 && a.bulk != 0);
+  const bool bulk = SPLIT || (OPT & REAL_BULK) != 0 || (XP == 0 && a.bulk != 0);
 
   const RealLayout lay = real_layout(xp, nthr, TY, has_src, (int)sizeof(T));
   const T* const ring = reinterpret_cast<const T*>(smraw + lay.ring);
@@ -321,11 +392,20 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
   V* const edge = reinterpret_cast<V*>(smraw + lay.edge);  // [2][nw][TY][3]: (own part of the receiver, left of the sender)
   uint64_t* const bar = reinterpret_cast<uint64_t*>(smraw + lay.bar);
 
-  const int x = tid;
-  const bool xact = x < n1;
-  const int xr = xact ? x : 0;
-  const int xmr = xr == 0 ? n1 - 1 : xr - 1;
-  const bool recv_shfl = lane < 31 && x + 1 < n1;  // the column on the right sits in this warp
+  if constexpr (SPLIT) {
+    // both blocks run or neither does: a block does not read the memory of one that has left
+    int* const flag = reinterpret_cast<int*>(smraw + lay.red);
+    if (tid == 0) *flag = skip ? 1 : 0;
+    cluster_sync();
+    const int leave = *flag | peer_load(flag, half ^ 1);
+    cluster_sync();
+    if (leave) return;
+  }
+  const int x = x0 + tid;
+  const bool xact = tid < nx;
+  const int xr = xact ? tid : 0;
+  const int xmr = SPLIT ? xr + XO - 1 : xr == 0 ? n1 - 1 : xr - 1;
+  const bool recv_shfl = lane < 31 && tid + 1 < nx;  // the column on the right sits in this warp
   // a warp's first column publishes its left-going sums, its last one its own sums (N1 is even, so
   // no lane is both)
   const bool at_edge = lane == 0 || (xact && !recv_shfl);
@@ -355,7 +435,9 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
     const int ib = want_ids ? (q & 1) : -1;
     const int sb = (has_src && pu > z0) ? q % 3 : -1;
     if (bulk) {
-      if (warp == 0) real_prefetch_bulk<T, TY>(a, lay, smraw, xp, y0, pu, q % 3, ib, pu - 1, sb, bar + q % 3);
+      if constexpr (SPLIT) {
+        if (warp == 0) real_prefetch_half<T, TY>(a, lay, smraw, xp, x0, nx, y0, pu, q % 3, ib, bar + q % 3);
+      } else if (warp == 0) real_prefetch_bulk<T, TY>(a, lay, smraw, xp, y0, pu, q % 3, ib, pu - 1, sb, bar + q % 3);
     } else {
       real_prefetch_async<T, TY>(a, lay, smraw, xp, y0, pu, q % 3, ib, pu - 1, sb);
     }
@@ -394,8 +476,8 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
     const bool out_plane = FORCE && p > z0;  // corner plane p - 1 belongs to this chunk
     const T* const rc = ring + sc * 3 * NR * xp;
     const T* const rp = ring + sp * 3 * NR * xp;
-    const T* const rcx = rc + xr;
-    const T* const rpx = rp + xr;
+    const T* const rcx = rc + xr + XO;
+    const T* const rpx = rp + xr + XO;
     const T* const rcl = rc + xmr;
     const T* const rpl = rp + xmr;
     const uint16_t* const idrow = sids + (q & 1) * (TY + 1) * xp + xr;
@@ -411,7 +493,7 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
     // and component); the other lanes' left columns come by shuffle
     T eS[2], eD[2];
     if constexpr (F64) {
-      const int xl = ((warp << 5) + n1 - 1) % n1;
+      const int xl = SPLIT ? (warp << 5) + XO - 1 : ((warp << 5) + n1 - 1) % n1;
 #pragma unroll
       for (int h = 0; h < (3 * NR + 31) / 32; ++h) {
         const int i = min(lane + 32 * h, 3 * NR - 1), o = ((i % 3) * NR + i / 3) * xp + xl;
@@ -532,18 +614,24 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
       }
       if (jj >= 2) frow += frstep;
     }
-    __syncthreads();
+    if (SPLIT) cluster_sync(); else __syncthreads();
     if (out_plane) {
       // the last column of every warp: its own part and the left-going part of the column to its right
       for (int i = tid; i < nw * TY * 3; i += nthr) {
         const int k = i % 3, wr = i / 3, w = wr / TY, r = wr - w * TY;
-        const int xe = min((w << 5) + 31, n1 - 1);
-        const int ws = (xe + 1 < n1) ? w + 1 : 0;
-        T F = ed[i].x + ed[(ws * TY + r) * 3 + k].y;
+        const int xe = min((w << 5) + 31, nx - 1);
+        const int ws = (xe + 1 < nx) ? w + 1 : 0;
+        T F;
+        if constexpr (SPLIT) {
+          const T* const left = &ed[(ws * TY + r) * 3 + k].y;
+          F = ed[i].x + (ws == 0 ? peer_load(left, half ^ 1) : *left);
+        } else {
+          F = ed[i].x + ed[(ws * TY + r) * 3 + k].y;
+        }
         if (has_src) F += (T)ssrc[(sc * 3 * TY + k * TY + r) * xp + xe];
         facc = ::fma(F, F, facc);
         if (a.fout != nullptr) {
-          const size_t o = k * rcomp + (size_t)(p - 1) * rplane + (size_t)(y0 + r) * n1 + xe;
+          const size_t o = k * rcomp + (size_t)(p - 1) * rplane + (size_t)(y0 + r) * n1 + x0 + xe;
           if (F64 && a.fout_f32) reinterpret_cast<float*>(a.fout)[o] = (float)F;
           else reinterpret_cast<T*>(a.fout)[o] = F;
         }
@@ -551,6 +639,7 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
     }
   }
   cp_async_wait_all();
+  if (SPLIT) cluster_sync();  // the other block may still read this one's sums
   if (timed_out) a.st->done = DONE_TIMEOUT;
   if (!FORCE) return;
   double acc[NRED];

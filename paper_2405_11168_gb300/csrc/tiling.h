@@ -24,7 +24,7 @@ inline long long greedy_end(long long yt, long long nz, long long slots, long lo
   return lo;
 }
 
-// z chunk and end time of an FP64 real-space pass in tiles of ty rows.  A warp needs 64 cycles of its
+// z chunk and end time of an FP64 real-space pass in yt tiles (or halves of them) of ty rows.  A warp needs 64 cycles of its
 // scheduler's FP64 lanes per instruction and nearly fills them by itself, so a block of w warps takes
 // (layers x voxel rows, both with their recomputed one) x max(1, w / 4) alone and an SM with more warps
 // than schedulers shares that rate.  While every block is resident, SM i runs blocks i, i + nsm, ...;
@@ -33,14 +33,14 @@ inline long long greedy_end(long long yt, long long nz, long long slots, long lo
 // rows, chunk 1 36 us (4 rows, chunk 4, which counting resident blocks alone chose: 117 us); 64^3 4 rows,
 // chunk 4 129 us (8 rows, chunk 4: 204 us); 128^3 4 rows, chunk 14 702 us (8 rows: 799); 256^3 8 rows,
 // chunk 27 4850 us.
-inline double pick_zchunk64(int n2, int n3, int ty, int warps, int per_sm, int nsm, int zc_min, int* zc_out) {
-  const long long yt = n2 / ty, rows = ty + 1, fixed = 2;  // start and reduction: about two voxel rows
+inline double pick_zchunk64(int yt, int n3, int ty, int warps, int per_sm, int nsm, int zc_min, int* zc_out) {
+  const long long rows = ty + 1, fixed = 2;  // start and reduction: about two voxel rows
   const int r = std::max(1, std::min(per_sm, (4 + warps - 1) / warps));  // blocks that fill an SM's schedulers
   double best = -1;
   for (int zc = zc_min; zc <= std::max(std::min(n3, 64), zc_min); ++zc) {
     const int nz = (n3 + zc - 1) / zc, last = n3 - (nz - 1) * zc;
     const long long t = (zc + 1) * rows + fixed, t_last = (last + 1) * rows + fixed;
-    const long long nblk = yt * nz, nfull = yt * (nz - 1);
+    const long long nblk = (long long)yt * nz, nfull = (long long)yt * (nz - 1);
     double end;
     int resident;
     if (nblk <= (long long)per_sm * nsm) {
@@ -88,7 +88,8 @@ template <typename T> int real_occupancy(bool iso, int n1, int ty, size_t smem) 
   memset(&a, 0, sizeof(a));
   a.n1 = n1;
   int n = 0;
-  if (launch_real<T>(a, iso, ty, MODE_FORCE, dim3(1), ((n1 + 31) / 32) * 32, smem, nullptr, &n) != cudaSuccess) {
+  if (launch_real<T>(a, iso, ty, MODE_FORCE, dim3(1), real_threads(sizeof(T) == 8, ty, n1), smem, nullptr, &n) !=
+      cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -97,25 +98,27 @@ template <typename T> int real_occupancy(bool iso, int n1, int ty, size_t smem) 
 
 // Shared memory of the real-space force pass.
 inline size_t real_bytes(bool f64, int n1, int ty, bool has_src) {
-  return real_layout(real_pitch(f64, ty, MODE_FORCE, n1), ((n1 + 31) / 32) * 32, ty, has_src, f64 ? 8 : 4).total;
+  return real_layout(real_pitch(f64, ty, MODE_FORCE, n1), real_threads(f64, ty, n1), ty, has_src, f64 ? 8 : 4).total;
 }
 
 // Row tile (8, 4 or 2 rows dividing n2, its planes within smem_limit; fixed_ty > 0: this one) and z chunk of
 // an FP64 real-space pass with the earliest modelled end.  Tiles of 8 rows need 255 registers, so rows of
-// more than 256 columns run 4 at most.  max_blocks > 0: at most this many blocks.
+// more than 256 columns run them in two halves (split_ok and real_rows_fit).  max_blocks > 0: at most this many blocks.
 inline void pick_tile64(bool iso, int n1, int n2, int n3, int fixed_ty, size_t smem_limit, int nsm, int max_blocks,
-                        int* ty_out, int* zc_out) {
+                        bool split_ok, int* ty_out, int* zc_out) {
   *ty_out = 2;
   *zc_out = std::min(n3, 16);
   double best = -1;
   for (int ty : {8, 4, 2}) {
-    if (n2 % ty != 0 || (fixed_ty > 0 ? ty != fixed_ty : ty == 8 && n1 > 256)) continue;
+    if (n2 % ty != 0 || (fixed_ty > 0 && ty != fixed_ty)) continue;
+    if (real_split(true, ty, n1) && !(split_ok && real_rows_fit(true, ty, n1))) continue;
     const size_t smem = real_bytes(true, n1, ty, false);
     if (smem > smem_limit) continue;
     const int occ = real_occupancy<double>(iso, n1, ty, smem);
     int zc = 0, zc_min = 1;
-    if (max_blocks > 0) zc_min = std::max(1, (int)(((long long)n3 * (n2 / ty) + max_blocks - n2 / ty) / std::max(1, max_blocks - n2 / ty)));
-    const double end = pick_zchunk64(n2, n3, ty, (n1 + 31) / 32, std::max(1, occ), nsm, std::min(zc_min, n3), &zc);
+    const int yt = n2 / ty * real_halves(true, ty, n1);
+    if (max_blocks > 0) zc_min = std::max(1, (int)(((long long)n3 * yt + max_blocks - yt) / std::max(1, max_blocks - yt)));
+    const double end = pick_zchunk64(yt, n3, ty, real_threads(true, ty, n1) / 32, std::max(1, occ), nsm, std::min(zc_min, n3), &zc);
     if (best < 0 || end < best) {
       best = end;
       *ty_out = ty;
