@@ -298,7 +298,7 @@ __device__ __forceinline__ void col_green_fixed(const ColArgs<T>& a, typename cp
 // 27.5 / 30.7 us; 192^3 with 24 values: 129 / 110)
 __host__ __device__ constexpr int col_max_threads(int nt, bool f64) { return nt > 0 ? nt : f64 ? 384 : 768; }
 __host__ __device__ constexpr int col_min_blocks(int nt, bool f64, bool wide) {
-  return nt > 0 ? (f64 ? 384 : wide ? 512 : 768) / nt : 1;
+  return nt > 0 ? (f64 ? 384 : wide ? 512 : nt > 256 ? 1024 : 768) / nt : 1;
 }
 
 // LF > 0: the transformed length is LF and the block has NT threads, both
