@@ -105,12 +105,13 @@ typedef struct {
   int col_state;        /* z pass + Green update: 0 = automatic, 1 = state read point by point (L2
                            prefetch), 2 = state tile copied to shared memory during the forward z
                            transform (twice the tile's shared memory); results do not change */
-  int col_pipe;         /* y passes at lengths 128, 256, 512 with the default tile: 0 = persistent
-                           blocks that copy the next tile while transforming the current one
-                           (default), 1 = one tile per block, 2 = persistent y passes and a
-                           persistent z pass (z lengths 128, 256, 512); results do not change */
-  int col_copy;         /* tile loads of the persistent y passes (y lengths 128, 256, 512) and of the
-                           z pass (z lengths 64, 128, 256, 512, state read point by point): 0 = tensor
+  int col_pipe;         /* y passes at lengths 128, 192, 256, 384, 512 with the default tile: 0 = automatic
+                           (default): persistent blocks that copy the next tile while transforming the
+                           current one in FP32 while the spectrum fits in L2, else one tile per block;
+                           1 = one tile per block, 2 = persistent y passes and a persistent z pass (at
+                           the same lengths); results do not change */
+  int col_copy;         /* tile loads of the column passes at lengths with a compile-time transform (the
+                           z pass: state read point by point): 0 = tensor
                            (TMA) copies where the driver encodes the tile map, else 16-byte cp.async
                            (default); 1 = cp.async; 2 = as 0, but HS_ERR_UNSUPPORTED_SIZE where such a
                            pass cannot have its map; results do not change.  A tensor copy that does

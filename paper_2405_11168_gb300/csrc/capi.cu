@@ -1512,8 +1512,13 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
     // the z pass stays one tile per block: its Green step waits on the state point by point, and
     // three resident blocks hide that better than two persistent ones (256^3 FP32: 0.228 against
     // 0.247 ms; the y passes gain, 0.095 against 0.101 ms)
+    // The y passes are persistent by default in FP32 while the spectrum stays in L2 (us, persistent against one
+    // tile per block: 192^3 34.2, 36.0; 256 x 128 x 256 36.6, 39.9); larger ones and FP64 run one tile per
+    // block (256^3 77.1, 73.2; 384^3 307, 294; 512 x 128 x 512 143, 131; FP64 128^3 141.5, 139.3; 256^3 1184, 1162).
+    const bool in_l2 = (size_t)3 * c->n3 * c->n2 * c->P * cs <= ((size_t)128 << 20);
     for (int axis = 1; axis <= (o.col_pipe == 2 ? 2 : 1) && o.col_pipe != 1 && !ext && nsm > 0; ++axis) {
       const int L = axis == 1 ? c->n2 : c->n3;
+      if (o.col_pipe == 0 && (c->f64 || !in_l2)) continue;
       if (!(axis == 1 ? c->fixed_y : c->fixed_z) || L < 128) continue;
       if (axis == 2 && c->zstate_smem) continue;  // the persistent z pass reads the state point by point
       // the tiles may arrive by tensor copies: room for their alignment and barriers

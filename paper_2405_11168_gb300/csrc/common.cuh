@@ -50,6 +50,15 @@ enum { DONE_RUNNING = 0, DONE_CONVERGED = 1, DONE_MAXITER = 2, DONE_DIVERGED = 3
 // 277 -> 442 us per evaluation, 256^3 FP32 650 -> 689.  So a pass calls it before its last transform.
 __device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pass_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// FP32 passes of a solve over 2^17 to 2^22 voxels launch as programmatic dependents of the kernel before them:
+// their blocks start and fill their twiddle tables while that kernel's last transforms run, and wait for its
+// results in pass_wait.  us per evaluation: 64^3 37.2 -> 34.5, 96^3 60.7 -> 58.5, 128^3 101.4 -> 97.5, but
+// 44^3 46.1 -> 47.5 (fewer blocks than SMs, some of which then get two), 192^3 328 -> 326 and 256^3 651 -> 655;
+// in FP64, whose passes need their blocks spread evenly over the SMs, 64^3 277 -> 326 and 128^3 1749 -> 1894.
+// The real-space pass is launched plainly for the same reason, and so are a batch's passes.
+template <typename T> __host__ __device__ constexpr bool pass_dependent(size_t zstride, size_t voxels) {
+  return sizeof(T) == 4 && zstride == 0 && voxels >= ((size_t)1 << 17) && voxels <= ((size_t)1 << 22);
+}
 
 // Batched launches (one launch over many solves of the same grid): item
 // blockIdx.z works in the workspace that starts zstride bytes after item

@@ -40,7 +40,7 @@ static cudaError_t col_one(const ColArgs<T>& a, dim3 g, int nthr, size_t smem, c
   }
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  return launch_pass<T>(k, a, (size_t)a.n1 * a.n2 * a.n3, g, nthr, smem, s);
+  return launch_pass(k, a, pass_dependent<T>(a.zstride, (size_t)a.n1 * a.n2 * a.n3), g, nthr, smem, s);
 }
 
 template <typename T, int CT, int LF = 0, int NT = 0>
@@ -98,7 +98,7 @@ static cudaError_t colp_one(const ColArgs<T>& a, dim3 g, size_t smem, cudaStream
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   if (occ != nullptr) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, NT, smem);
-  return launch_pass<T>(k, a, (size_t)a.n1 * a.n2 * a.n3, g, NT, smem, s);
+  return launch_pass(k, a, pass_dependent<T>(a.zstride, (size_t)a.n1 * a.n2 * a.n3), g, NT, smem, s);
 }
 
 // the persistent column pass at a fixed length: launch it, or (occ) its blocks per SM
@@ -130,7 +130,7 @@ static cudaError_t row_launch(const RowArgs<T>& a, dim3 nb, int nthr, size_t sme
   auto k = k_row<T, MODE, LF, BATCH>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  return launch_pass<T>(k, a, (size_t)a.n1 * a.nrows / 3, nb, nthr, smem, s);
+  return launch_pass(k, a, pass_dependent<T>(a.zstride, (size_t)a.n1 * a.nrows / 3), nb, nthr, smem, s);
 }
 
 template <typename T, int MODE, int LF = 0>

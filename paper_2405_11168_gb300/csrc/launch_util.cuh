@@ -37,14 +37,9 @@ template <typename K> static cudaError_t set_smem(K kernel, size_t smem) {
   return e;
 }
 
-// Launch of a transform pass.  FP32 passes of a solve over at most 2^22 voxels launch as programmatic
-// dependents of the kernel before them: their blocks start and fill their twiddle tables while that kernel's
-// last transforms run (pass_begin), and wait for its results in pass_wait.  us per evaluation: 64^3 37.2 ->
-// 34.5, 96^3 60.7 -> 58.5, 128^3 101.4 -> 97.5, but 192^3 328 -> 326 and 256^3 651 -> 655; in FP64, whose passes
-// need their blocks spread evenly over the SMs, 64^3 277 -> 326 and 128^3 1749 -> 1894.  The real-space pass
-// is launched plainly for the same reason (44^3 46 -> 48), and so are a batch's (32^3 to 128^3 51.8 -> 52.3 ms).
-template <typename T, typename K, typename A>
-static cudaError_t launch_pass(K kernel, const A& a, size_t voxels, dim3 g, int nthr, size_t smem, cudaStream_t s) {
+// Launch of a transform pass, plainly or as a programmatic dependent of the kernel before it.
+template <typename K, typename A>
+static cudaError_t launch_pass(K kernel, const A& a, bool dependent, dim3 g, int nthr, size_t smem, cudaStream_t s) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -54,7 +49,7 @@ static cudaError_t launch_pass(K kernel, const A& a, size_t voxels, dim3 g, int 
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &at;
-  cfg.numAttrs = sizeof(T) == 4 && a.zstride == 0 && voxels <= ((size_t)1 << 22) ? 1 : 0;
+  cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 

@@ -147,26 +147,36 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
   C* const tws = reinterpret_cast<C*>(smraw + L.tws);
   const bool bload = LF > 0 && (L.rowbytes & 15) == 0;
   uint64_t* sbar = reinterpret_cast<uint64_t*>(smraw + L.bar);
-  if constexpr (LF > 0) stage_twiddles<RowPlan<LF>>(tws, a.tw, tid, nthr);
-  if (bload && tid == 0) {
-    mbar_init(sbar, 1);
-    mbar_init(sbar + 1, 1);
-    mbar_init_fence();
+  // The stopping test of this evaluation runs beside the row transforms instead of at the end of the
+  // real-space pass, where the whole chip waited for one block (12 of 31 us at 64^3).  A done flag
+  // that it sets is seen by the next kernels; blocks of this one that see it early skip rows nobody reads.
+  const int nfin = (MODE == ROW_R2C && a.nparts > 0) ? 1 : 0;
+  const bool fin = MODE == ROW_R2C && nfin && blockIdx.x == 0;
+  // a dependent fills the table before the wait (read after the barrier that opens the first batch)
+  const bool early = !BATCH && pass_dependent<T>(a.zstride, (size_t)n1 * a.nrows / 3);
+  if constexpr (LF > 0) {
+    if (early && !fin) stage_twiddles<RowPlan<LF>>(tws, a.tw, tid, nthr);
   }
-  if (LF > 0) __syncthreads();
   pass_wait();
   // In the pass that takes the stopping test the done flag may change while blocks start: the block
   // decides as one.
   bool skip = a.st->retired || (a.skip_if_done && a.st->done);
   if (MODE == ROW_R2C) skip = __syncthreads_or(skip);
   if (skip) return;
-  // The stopping test of this evaluation runs beside the row transforms instead of at the end of the
-  // real-space pass, where the whole chip waited for one block (12 of 31 us at 64^3).  A done flag
-  // that it sets is seen by the next kernels; blocks of this one that see it early skip rows nobody reads.
-  const int nfin = (MODE == ROW_R2C && a.nparts > 0) ? 1 : 0;
-  if (MODE == ROW_R2C && nfin && blockIdx.x == 0) {
+  if (fin) {
     finalize_partials(a.nparts, a.partials, a.st, a.hist, reinterpret_cast<double*>(smraw));
     return;
+  }
+  if (bload) {
+    if (tid == 0) {
+      mbar_init(sbar, 1);
+      mbar_init(sbar + 1, 1);
+      mbar_init_fence();
+    }
+    __syncthreads();
+  }
+  if constexpr (LF > 0) {
+    if (!early) stage_twiddles<RowPlan<LF>>(tws, a.tw, tid, nthr);
   }
   const int blk = (int)blockIdx.x - nfin, nblk = (int)gridDim.x - nfin;
   const int T8 = LF > 0 ? RowPlan<(LF > 0 ? LF : 64)>::T : (n1 + kE - 1) / kE;  // threads per sequence
