@@ -54,7 +54,14 @@ def test_wide_rows(hs, n1):
     check(hs, (n1, 8, 6), 0, eigen=True)
 
 
-def check(hs, grid, ytile, eigen):
+@pytest.mark.parametrize("n1", [288, 320, 352, 512])
+def test_wide_rows_in_halves(hs, n1):
+    """Tiles of 8 FP64 rows of more than 256 columns run as two blocks of a cluster (partial warps at 288 to 352):
+    the FP64 sweep of the refined precision, with a wrapped first row and tiles on both sides."""
+    check(hs, (n1, 16, 6), 8, eigen=(n1 == 320), precisions=(hs.HS_FP32_REFINED,))
+
+
+def check(hs, grid, ytile, eigen, precisions=None):
     n1, n2, n3 = grid
     for law in ("iso", "aniso"):
         ids = synth.random_phase_map(grid, 3, seed=n1 + ytile)
@@ -70,6 +77,8 @@ def check(hs, grid, ytile, eigen):
         want = T.voigt_from_tensor(ref.eps), T.voigt_from_tensor(ref.sig)
         for prec, tol, dtype in ((hs.HS_FP64, 1e-10, torch.float64), (hs.HS_FP32, 1e-5, torch.float32),
                                  (hs.HS_FP32_REFINED, 1e-5, torch.float32)):
+            if precisions is not None and prec not in precisions:
+                continue
             kw = dict(C0=C0, precision=prec, ytile=ytile, zchunk=4, out_f32=int(dtype == torch.float32))
             if prec == hs.HS_FP64 and ytile == 8 and n1 == 256:
                 with pytest.raises(hs.HSError):  # a tile that is too large stays refused
