@@ -54,10 +54,11 @@ def test_wide_rows(hs, n1):
     check(hs, (n1, 8, 6), 0, eigen=True)
 
 
-@pytest.mark.parametrize("n1", [288, 320, 352, 512])
+@pytest.mark.parametrize("n1", [288, 320, 352])
 def test_wide_rows_in_halves(hs, n1):
     """Tiles of 8 FP64 rows of more than 256 columns run as two blocks of a cluster (partial warps at 288 to 352):
-    the FP64 sweep of the refined precision, with a wrapped first row and tiles on both sides."""
+    the FP64 sweep of the refined precision, with a wrapped first row and tiles on both sides.  (An explicit
+    tile of 8 rows at 512 columns is refused: the FP32 pass has no room for it.)"""
     check(hs, (n1, 16, 6), 8, eigen=(n1 == 320), precisions=(hs.HS_FP32_REFINED,))
 
 
