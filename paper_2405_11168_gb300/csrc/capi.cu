@@ -1510,8 +1510,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
     const bool ext = hs::plan_ext(c->plan[1]) || hs::plan_ext(c->plan[2]);
     const int xtiles = (c->nh + c->ct - 1) / c->ct;
     // the z pass stays one tile per block: its Green step waits on the state point by point, and
-    // three resident blocks hide that better than two persistent ones (256^3 FP32: 0.228 against
-    // 0.247 ms; the y passes gain, 0.095 against 0.101 ms)
+    // three resident blocks hide that better than two persistent ones (256^3 FP32: 0.185 against 0.255 ms)
     // The y passes are persistent by default in FP32 while the spectrum stays in L2 (us, persistent against one
     // tile per block: 192^3 34.2, 36.0; 256 x 128 x 256 36.6, 39.9); larger ones and FP64 run one tile per
     // block (256^3 77.1, 73.2; 384^3 307, 294; 512 x 128 x 512 143, 131; FP64 128^3 141.5, 139.3; 256^3 1184, 1162).
