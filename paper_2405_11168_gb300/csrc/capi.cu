@@ -578,6 +578,7 @@ template <typename T> void fill_march_common(hs_ctx* c, hs::MarchArgs<T>& a) {
 template <typename T> void set_real_rows(hs::MarchArgs<T>& a, int ty, int mode) {
   a.xp = hs::real_pitch(sizeof(T) == 8, ty, mode, a.n1);
   a.bulk = (a.n1 % 8 == 0) ? 1 : 0;
+  a.sum_planes = hs::sum_planes(a.n2 / ty, a.n3);
 }
 
 template <typename T> void fill_col(hs_ctx* c, hs::ColArgs<T>& a, void* buf, int axis) {

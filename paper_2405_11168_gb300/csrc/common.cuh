@@ -193,19 +193,17 @@ __device__ inline void finalize_eval(DevStatus* st, double* hist, double sum) {
   }
 }
 
-// Sums of 8 values per thread over the block, in a fixed order, valid in lanes 0..7 of warp 0 (lane v:
-// value v).  A warp sums its 32 x 8 values in 9 additions per lane instead of 8 x 5: each of the first
-// three exchanges also halves the values a lane keeps.  (FP64 additions run at 2 lanes per SM and
-// clock, so the plain form cost each block of a pass about 2 us.)  scratch: kReduceScratch bytes of
-// shared memory.  Every thread of the block must call it.
-__device__ inline double block_sum8(const double (&acc)[8], double* scratch) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x + 31) >> 5;
-  double v[4];
+// Sums of 8 values per thread over the warp, in a fixed order; lane l returns value l / 4.  9 additions per
+// lane instead of 8 x 5: each of the first three exchanges also halves the values a lane keeps.  (FP64
+// additions run at 2 lanes per SM and clock, so the plain form cost each block of a pass about 2 us.)
+template <typename T> __device__ __forceinline__ T warp_sum8(const T (&acc)[8]) {
+  const int lane = threadIdx.x & 31;
+  T v[4];
   {
     const bool up = (lane & 16) != 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const double keep = up ? acc[4 + i] : acc[i], send = up ? acc[i] : acc[4 + i];
+      const T keep = up ? acc[4 + i] : acc[i], send = up ? acc[i] : acc[4 + i];
       v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
     }
   }
@@ -213,15 +211,22 @@ __device__ inline double block_sum8(const double (&acc)[8], double* scratch) {
     const bool up = (lane & 8) != 0;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const double keep = up ? v[2 + i] : v[i], send = up ? v[i] : v[2 + i];
+      const T keep = up ? v[2 + i] : v[i], send = up ? v[i] : v[2 + i];
       v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
     }
   }
   const bool up = (lane & 4) != 0;
-  const double keep = up ? v[1] : v[0], send = up ? v[0] : v[1];
-  double s = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  const T keep = up ? v[1] : v[0], send = up ? v[0] : v[1];
+  T s = keep + __shfl_xor_sync(0xffffffffu, send, 4);
   s += __shfl_xor_sync(0xffffffffu, s, 2);
   s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
+}
+
+// Sums over the block of the warps' sums (warp_sum8), valid in lanes 0..7 of warp 0 (lane v: value v).
+// scratch: kReduceScratch bytes of shared memory.  Every thread of the block must call it.
+__device__ inline double block_sum8(double s, double* scratch) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x + 31) >> 5;
   if ((lane & 3) == 0) scratch[warp * 8 + (lane >> 2)] = s;
   __syncthreads();
   double t = 0;
@@ -248,12 +253,11 @@ __device__ inline bool last_block_arrived(DevStatus* st, unsigned int nblk) {
   return am_last;
 }
 
-// Block-sum NRED doubles (fixed order) and publish them as this block's partials.  scratch:
-// kReduceScratch bytes of shared memory.
-__device__ inline void publish_partials(const double (&acc)[NRED], double* partials, double* scratch) {
+// Sum the warps' sums (warp_sum8 of NRED values and a zero) over the block and publish them as its partials.
+// scratch: kReduceScratch bytes of shared memory.
+__device__ inline void publish_partials(double warp_sum, double* partials, double* scratch) {
   const int bid = blockIdx.y * gridDim.x + blockIdx.x;
-  const double a8[8] = {acc[0], acc[1], acc[2], acc[3], acc[4], acc[5], acc[6], 0.0};
-  const double s = block_sum8(a8, scratch);
+  const double s = block_sum8(warp_sum, scratch);
   if (threadIdx.x < 8) partials[(size_t)bid * kPartStride + threadIdx.x] = s;
 }
 
@@ -277,16 +281,16 @@ __device__ inline void finalize_partials(int nblk, const double* partials, DevSt
       if (v < 3) a8[2 * v + 1] += d[v].y;
     }
   }
-  const double t = block_sum8(a8, scratch);
+  const double t = block_sum8(warp_sum8(a8), scratch);
   if (threadIdx.x < 32) finalize_eval(st, hist, t);
 }
 
 // Publish this block's partials; the last block to arrive takes the sum and the
 // stopping test (passes that no kernel of the same evaluation follows).
-__device__ inline void reduce_and_finalize(const double (&acc)[NRED], double* partials, DevStatus* st,
-                                           double* hist, double* scratch) {
+__device__ inline void reduce_and_finalize(double warp_sum, double* partials, DevStatus* st, double* hist,
+                                           double* scratch) {
   const int nblk = gridDim.x * gridDim.y;
-  publish_partials(acc, partials, scratch);
+  publish_partials(warp_sum, partials, scratch);
   if (!last_block_arrived(st, (unsigned)nblk)) return;
   finalize_partials(nblk, partials, st, hist, scratch);
 }

@@ -56,6 +56,7 @@ template <typename T> struct MarchArgs {
   int xp;                // k_real: row pitch in shared memory (a multiple of 8, >= n1)
   int defer;             // k_real: 1 = the forward row pass that follows sums the partials and takes the stopping test
   int bulk;              // k_real: 1 = planes arrive by bulk copies (n1 a multiple of 8, inputs 16-byte aligned)
+  int sum_planes;        // k_real, FP32: planes whose sums a thread keeps in one chain of FP32 additions
   int skip_if_done;
   const double* Edev;    // not null: the macroscopic strain is read here (applied-stress control)
   const T* sig0;         // not null: lambda(ph) : eps0(ph) per phase, Voigt [nphase][6] (eigenstrain)
@@ -634,11 +635,12 @@ __global__ void __launch_bounds__(512) k_march(const MarchArgs<T> a, const MAT m
   }
   cp_async_wait_all();
   if (MODE != MODE_FORCE) return;
-  double acc[NRED];
+  double acc[8];
 #pragma unroll
   for (int i = 0; i < 6; ++i) acc[i] = (double)sacc[i];
   acc[6] = (double)facc;
-  reduce_and_finalize(acc, a.partials, a.st, a.hist, red);
+  acc[7] = 0.0;
+  reduce_and_finalize(warp_sum8(acc), a.partials, a.st, a.hist, red);
 }
 
 }  // namespace hs

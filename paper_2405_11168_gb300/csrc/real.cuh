@@ -123,6 +123,8 @@ template <typename T> struct RealAniso {
   }
 };
 
+constexpr int kSumBytes = 56;  // RealSums, per thread: three float4 (two high parts, two low parts), one float2
+
 // Shared memory of k_real.  xp: row pitch (elements); host and device use the same function.
 struct RealLayout {
   size_t ring, ids, src, edge, red, bar, total;
@@ -139,13 +141,69 @@ __host__ __device__ inline RealLayout real_layout(int xp, int nthr, int ty, bool
   off += hs_align16(has_src ? (size_t)4 * 3 * 3 * ty * xp : 0);
   L.edge = off;  // [2][nwarps][ty][3] x (own, left)
   off += hs_align16((size_t)2 * 2 * tsize * (nthr / 32) * ty * 3);
-  L.red = off;
-  off += kReduceScratch;
+  L.red = off;   // block sums; FP32: before them the threads' running sums (RealSums)
+  off += tsize == 4 && (size_t)kSumBytes * nthr > kReduceScratch ? (size_t)kSumBytes * nthr : kReduceScratch;
   L.bar = off;
   off += 32;
   L.total = off;
   return L;
 }
+
+// A thread's running sums of the FP32 pass, 6 stress components and |F|^2, in shared memory as unevaluated
+// pairs (high, low) of floats.  FP32 registers hold the terms of a few planes only (MarchArgs::sum_planes)
+// and are then added here, the rounding error of each addition kept in the low part (Knuth's two-sum), so a
+// sum's accuracy does not depend on the chunk.  One FP32 chain over a whole chunk (32 planes of 4 rows at 192^3)
+// left up to 1.7e-6 in the mean stress of a uniform field.
+struct RealSums {
+  using P = Pair<float>;
+  float4* s;  // [3][nthr]
+  float2* f;  // [nthr]
+  __device__ __forceinline__ RealSums(unsigned char* base, int tid, int nthr)
+      : s(reinterpret_cast<float4*>(base) + tid), f(reinterpret_cast<float2*>(base + (size_t)48 * nthr) + tid) {}
+  __device__ __forceinline__ void clear(int nthr) const {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s[i * nthr] = make_float4(0.f, 0.f, 0.f, 0.f);
+    *f = make_float2(0.f, 0.f);
+  }
+  // the registers' sums go in and start again from 0
+  __device__ __forceinline__ void take(float (&sacc)[6], float& facc, int nthr) const {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      float4 v = s[i * nthr];
+      two_sum(v, make_float2(sacc[2 * i], sacc[2 * i + 1]));
+      s[i * nthr] = v;
+      sacc[2 * i] = sacc[2 * i + 1] = 0.f;
+    }
+    float4 v = make_float4(f->x, 0.f, f->y, 0.f);
+    two_sum(v, make_float2(facc, 0.f));
+    *f = make_float2(v.x, v.z);
+    facc = 0.f;
+  }
+  // (v.x, v.y) + b with the rounding errors added to (v.z, v.w)
+  static __device__ __forceinline__ void two_sum(float4& v, float2 b) {
+    auto sub = [](float2 a, float2 c) { return __ffma2_rn(c, make_float2(-1.f, -1.f), a); };
+    const float2 hi = make_float2(v.x, v.y), t = P::add(hi, b), z = sub(t, hi);
+    const float2 lo = P::add(P::add(sub(hi, sub(t, z)), sub(b, z)), make_float2(v.z, v.w));
+    v = make_float4(t.x, t.y, lo.x, lo.y);
+  }
+  // a warp's sums (lane l: value l / 4): the high parts in FP64, the low parts, which are 2^-24 of them, in FP32
+  // (an FP64 conversion costs a warp 64 cycles).  An infinite high part has no low part.
+  __device__ __forceinline__ double warp_total(bool xact, int nthr) const {
+    double h[8];
+    float l[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 v = i < 3 ? s[i * nthr] : make_float4(f->x, 0.f, f->y, 0.f);
+      const bool in = xact || i == 3;
+      h[2 * i] = in ? (double)v.x : 0.0;
+      h[2 * i + 1] = in && i < 3 ? (double)v.y : 0.0;
+      l[2 * i] = in && v.z == v.z ? v.z : 0.f;
+      l[2 * i + 1] = in && i < 3 && v.w == v.w ? v.w : 0.f;
+    }
+    const double scale = (threadIdx.x & 31) < 24 ? 0.5 / (double)kTabScale<float> : 1.0;
+    return scale * (warp_sum8(h) + (double)warp_sum8(l));
+  }
+};
 
 // Copy of one plane by warp 0: u rows y0 - 1 .. y0 + TY of corner plane pu into ring slot `slot`, the id
 // rows y0 .. y0 + TY of voxel plane pu into ids buffer ib (ib < 0: none), the source rows of output
@@ -339,6 +397,11 @@ __device__ __forceinline__ void real_prefetch_async(const MarchArgs<T>& a, const
   cp_async_commit();
 }
 
+// Resident blocks per SM that the registers of an FP32 pass with bulk copies must allow: 16 warps, 12 for blocks of up
+// to 128 threads, whose values then all stay in (up to 168) registers.  16 for those too: 128^3 34.6 -> 30.9 us, but
+// 64^3 14.4 -> 15.0, 96 x 192 x 384 95.5 -> 98.5, 64 x 256 x 256 48.1 -> 51.6.  0: left to the compiler.
+__host__ __device__ constexpr int real_min_blocks(int nt, bool bulk) { return !bulk ? 0 : nt >= 256 ? 512 / nt : 384 / nt; }
+
 // One block: corner rows y0 .. y0 + TY - 1 (TY divides N2) of one z chunk, thread x <-> column x.
 // XP > 0: compile-time row pitch in shared memory (N1 <= XP), so that row offsets are immediates;
 // XP = 0: a.xp.  NT: the largest block (its registers).  OPT: what the launch has, as compile-time
@@ -351,13 +414,17 @@ __device__ __forceinline__ void real_prefetch_async(const MarchArgs<T>& a, const
 // and completes corner plane p - 1.  One block barrier per step: it publishes the left-going sums of
 // each warp's first column, which the previous warp's last column needs, and frees ring slot p - 2.
 //
+// FP32 sums: sacc and facc hold the terms of sum_planes planes, then RealSums takes them.  The groups are a loop
+// around the steps; the same addition behind a test in each step cost the whole pass 11% (256^3: 174 -> 194 us, nested 175),
+// because the compiler then kept the sums and the test live through the step.
+//
 // REAL_SPLIT (FP64, more than 256 columns): the two blocks of a cluster take half the columns each, the barrier
 // of a step is the cluster's, and a half's last column reads the sums of the other half's first one from
 // that block's shared memory.  One block of 512 threads has 128 registers and shared memory for tiles of 2
 // rows, which compute 3 voxel rows for 2; halves of 256 run 8 rows with 255 registers: FP64 sweep of 512^3, 21-constant
 // law, 64.1 -> 51.6 ms.
 template <typename T, int TY, class MAT, int MODE, int XP, int NT, int OPT, bool BATCH>
-__global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT mat_) {
+__global__ void __launch_bounds__(NT, real_min_blocks(NT, (OPT & REAL_BULK) != 0)) k_real(const MarchArgs<T> a_, const MAT mat_) {
   using P = Pair<T>;
   using V = typename P::V;
   constexpr int NR = TY + 2;
@@ -420,6 +487,9 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
 #pragma unroll
   for (int i = 0; i < 6; ++i) sacc[i] = 0;
   T facc = 0;
+  constexpr bool SUMS = !F64 && FORCE;  // FP32: the sums of several planes are kept in RealSums
+  const RealSums sums(smraw + lay.red, tid, nthr);
+  if constexpr (SUMS) sums.clear(nthr);
   T E4[6];  // 4 x engineering macro strain
 #pragma unroll
   for (int i = 0; i < 6; ++i) E4[i] = (i < 3 ? T(4) : T(8)) * macro_E(a, i);
@@ -455,7 +525,13 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
   prefetch(z0, true);
   if (bulk) timed_out |= !mbar_wait(bar, 0);
 
-  for (int p = z0; p <= pend; ++p) {
+  // steps in groups of sum_planes (FP32), after which the registers' sums move on
+  const int group = SUMS ? a.sum_planes : pend - z0 + 1;
+  auto group_end = [&]() {
+    if constexpr (SUMS) sums.take(sacc, facc, nthr);
+  };
+  for (int p = z0; p <= pend; group_end())
+  for (const int pe = min(p + group - 1, pend); p <= pe; ++p) {
     const int q = p - z0 + 1;
     const int sc = q % 3, sp = (q + 2) % 3;
     if (p < pend) {
@@ -642,13 +718,21 @@ __global__ void __launch_bounds__(NT) k_real(const MarchArgs<T> a_, const MAT ma
   if (SPLIT) cluster_sync();  // the other block may still read this one's sums
   if (timed_out) a.st->done = DONE_TIMEOUT;
   if (!FORCE) return;
-  double acc[NRED];
+  double wsum;
+  if constexpr (SUMS) {
+    wsum = sums.warp_total(xact, nthr);
+    __syncthreads();  // the block sums use the same memory
+  } else {
+    double acc[8];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) acc[i] = xact ? (0.5 / (double)kTabScale<T>) * (double)sacc[i] : 0.0;
-  acc[6] = (double)facc;
+    for (int i = 0; i < 6; ++i) acc[i] = xact ? (0.5 / (double)kTabScale<T>) * (double)sacc[i] : 0.0;
+    acc[6] = (double)facc;
+    acc[7] = 0.0;
+    wsum = warp_sum8(acc);
+  }
   double* const red = reinterpret_cast<double*>(smraw + lay.red);
-  if (a.defer) publish_partials(acc, a.partials, red);
-  else reduce_and_finalize(acc, a.partials, a.st, a.hist, red);
+  if (a.defer) publish_partials(wsum, a.partials, red);
+  else reduce_and_finalize(wsum, a.partials, a.st, a.hist, red);
 }
 
 }  // namespace hs

@@ -62,6 +62,11 @@ inline double pick_zchunk64(int yt, int n3, int ty, int warps, int per_sm, int n
   return best;
 }
 
+// Planes whose sums a thread of the FP32 real-space pass keeps in FP32 registers before they go to its
+// two-float sums: 4 (at most 16 stress values per chain), fewer on small grids, whose chunks are short and whose
+// passes wait for latency and not for instructions, so that the addition is free there.
+inline int sum_planes(int yt, int n3) { return (int)std::max(1LL, std::min(4LL, (long long)yt * n3 / 1024)); }
+
 // z chunk of the FP32 real-space pass.  With w warps on an SM a plane of a block takes about 1.15 + 0.1 w
 // (latency, then issue slots), so a chunk costs that for its planes, the recomputed one and a start worth
 // 1.3 more, for every full wave of the resident blocks and for what is left over.  Measured at 128^3 (us): chunks 4 / 5 / 8 / 10 / 13 / 16 / 32: 41.9 / 36.8 / 43.0 /
