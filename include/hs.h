@@ -124,12 +124,14 @@ typedef struct {
 hs_status hs_default_options(hs_options* opt);
 
 /* Autotuner with a process-wide plan cache (no counterpart in the paper: it picks launch
- * shapes, not numerics).  Times `iters` evaluations of each candidate tiling of the
+ * shapes, not numerics).  Times `iters` evaluations of the automatic tiling (ytile = 0, zchunk = 0)
+ * and of each candidate tiling of the
  * real-space and FFT passes (y tile 2/4/8 x z chunk, then the wider column tile and the z
- * pass's col_state) with
+ * pass's col_state), which has to be 2% faster to replace it, with
  * CUDA events on `stream`, using the caller's workspace (hs_workspace_size bytes for
  * `base`), and writes the fastest options to *best (*best_ms: ms per evaluation, or -1
- * when the plan came from the cache).  Results do not depend on the tiling beyond
+ * when the plan came from the cache).  The automatic tiling is returned as its rows and planes where
+ * these options give exactly it, else as 0.  Results do not depend on the tiling beyond
  * rounding order.  Keyed by grid, precision and whether all phases are isotropic.
  * Errors: as hs_create / hs_solve; HS_ERR_CUDA if no candidate ran. */
 hs_status hs_autotune(const int grid[3], const hs_material* m, const hs_options* base, void* workspace,

@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <map>
 #include <mutex>
 #include <string>
@@ -508,9 +509,10 @@ size_t march_smem(int n1, int ty, bool f64, int mode, bool real, bool has_src = 
   return hs::march_layout(n1, pitch_of(n1 / 2 + 1, f64), nthr, ty, mode, has_src, ts).total;
 }
 
-// Largest shared memory of a real-space tile that an explicit ytile may ask for: the planes, two source
-// buffers, ids and edges of the tile.  (The pass itself keeps a third source buffer; a tile that only
-// just fits runs with half its rows.)
+// The limit of an explicit ytile, one for every precision and mode: the planes, two source buffers, ids and
+// edges of a tile.  (What a pass needs may differ: an FP32 tile that only just fits runs with half its rows, for the
+// third source buffer and the running sums; an FP64 pass has no source, and the automatic choice takes FP64 tiles
+// that are not offered here.)
 size_t real_tile_bytes(int n1, int ty, bool f64) {
   const size_t ts = f64 ? 8 : 4, nw = (n1 + 31) / 32, nr = ty + 2;
   auto al = [](size_t x) { return hs::hs_align16(x); };
@@ -1942,8 +1944,8 @@ hs_status hs_autotune(const int grid[3], const hs_material* m_in, const hs_optio
       return HS_OK;
     }
   }
-  // candidates: y tile x z chunk of the real-space pass (blocks targeted at 512 .. 4096), then
-  // the column tile width and the z pass's state staging
+  // candidates beside the automatic choice: y tile x z chunk of the real-space pass (blocks targeted at
+  // 512 .. 4096), then the column tile width and the z pass's state staging
   std::vector<hs_options> cands;
   for (int ty : {2, 4, 8}) {
     if (grid[1] % ty != 0) continue;
@@ -1966,6 +1968,15 @@ hs_status hs_autotune(const int grid[3], const hs_material* m_in, const hs_optio
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return fail(nullptr, HS_ERR_CUDA, "event create");
+  using Tiling = std::array<int, 4>;  // rows and planes of the real-space pass and of the FP64 sweep
+  auto tiling_of = [&](const hs_options& o, Tiling* t) -> hs_status {
+    hs_ctx* c = nullptr;
+    const hs_status st = hs_create(&c, grid, m, nullptr, &o, workspace, workspace_bytes, stream);
+    if (st != HS_OK) return st;
+    *t = {c->ty, c->zc, c->ty64, c->zc64};
+    hs_destroy(c);
+    return HS_OK;
+  };
   auto time_one = [&](const hs_options& o, double* ms) -> hs_status {
     hs_ctx* c = nullptr;
     hs_status st = hs_create(&c, grid, m, nullptr, &o, workspace, workspace_bytes, stream);
@@ -1988,30 +1999,51 @@ hs_status hs_autotune(const int grid[3], const hs_material* m_in, const hs_optio
   };
   double best_t = 1e300;
   hs_options win = b;
-  for (const hs_options& o : cands) {
+  // the plan to beat is the automatic choice, which the block targets need not hit; a plan has to be faster
+  // than the one before it by more than two timings of one plan differ
+  auto try_plan = [&](const hs_options& o) {
     double t = 0;
-    if (time_one(o, &t) == HS_OK && t < best_t) {
+    if (time_one(o, &t) == HS_OK && t < 0.98 * best_t) {
       best_t = t;
       win = o;
     }
+  };
+  hs_options dflt = b;
+  dflt.ytile = dflt.zchunk = 0;
+  try_plan(dflt);
+  if (best_t < 1e300) {
+    // as explicit numbers where these give the same tiling (an explicit ytile also sets the FP64 sweep's
+    // rows, and the widest FP64 rows are not offered as one)
+    Tiling want, got;
+    hs_options o = dflt;
+    if (tiling_of(dflt, &want) == HS_OK) {
+      o.ytile = want[0];
+      o.zchunk = want[1];
+      if (tiling_of(o, &got) == HS_OK && got == want) win = o;
+    }
+  }
+  double cand_t = 1e300;
+  hs_options cand = b;
+  for (const hs_options& o : cands) {
+    double t = 0;
+    if (time_one(o, &t) == HS_OK && t < cand_t) {
+      cand_t = t;
+      cand = o;
+    }
+  }
+  if (cand_t < 0.98 * best_t) {
+    best_t = cand_t;
+    win = cand;
   }
   {
     hs_options o = win;  // the wider column tile
     o.col_tile = (b.precision == HS_FP64) ? 8 : 16;
-    double t = 0;
-    if (time_one(o, &t) == HS_OK && t < best_t) {
-      best_t = t;
-      win = o;
-    }
+    try_plan(o);
   }
   for (int cs : {1, 2}) {
     hs_options o = win;  // the z pass's state staging
     o.col_state = cs;
-    double t = 0;
-    if (time_one(o, &t) == HS_OK && t < best_t) {
-      best_t = t;
-      win = o;
-    }
+    try_plan(o);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
