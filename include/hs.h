@@ -167,9 +167,9 @@ hs_status hs_create_sized(hs_ctx** out, const int grid[3], const hs_material* m,
                           const hs_options* opt, int layout_nphase, void* workspace, size_t workspace_bytes,
                           void* stream);
 
-/* Bind a context to another microstructure of the same grid, keeping its workspace, launch
- * configuration and captured iteration graphs resident (a serving slot reused for a new
- * request).  The phase ids and table are copied in (m as for hs_create; at most the phase count
+/* Bind a context to another microstructure of the same grid, keeping its workspace, options
+ * and captured iteration graphs resident (a serving slot reused for a new
+ * request); its launch shapes are those of a context created with that microstructure.  The phase ids and table are copied in (m as for hs_create; at most the phase count
  * the layout was sized for) and the reference medium is chosen again (C0, or the policy when
  * NULL).  Captured graphs stay valid when the reference medium is isotropic and the phases stay
  * isotropic (or stay anisotropic); otherwise the next solve captures them again.  Removes any

@@ -1827,6 +1827,13 @@ hs_status hs_set_material(hs_ctx* c, const hs_material* m, const double C0[36]) 
   if (!same_kernels) drop_graphs(c);
   c->nphase = t->nphase;
   c->iso = t->iso;
+  // the tiling of a context created with this material: it follows the law's kernels
+  c->ty = t->ty;
+  c->zc = t->zc;
+  c->grid_m = t->grid_m;
+  c->ty64 = t->ty64;
+  c->zc64 = t->zc64;
+  c->grid_m64 = t->grid_m64;
   c->table = t->table;
   memcpy(c->C0, t->C0, sizeof(c->C0));
   memcpy(c->G6, t->G6, sizeof(c->G6));
