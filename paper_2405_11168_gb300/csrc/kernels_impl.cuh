@@ -139,9 +139,9 @@ static cudaError_t row_one(const RowArgs<T>& a, dim3 nb, int nthr, size_t smem, 
   return row_launch<T, MODE, LF, false>(a, nb, nthr, smem, s);
 }
 
-template <typename T, int MODE, int LF = 0>
+template <typename T, int MODE, int LF = 0, bool BATCH = false>
 static cudaError_t row_occ_one(int nthr, size_t smem, int* n) {
-  auto k = k_row<T, MODE, LF>;
+  auto k = k_row<T, MODE, LF, BATCH>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, nthr, smem);
@@ -295,7 +295,7 @@ __global__ void k_state_import(const double2* in, typename cplx_t<T>::type* S, s
   case LEN: return col_ct<float, 8, LEN, col_block(ColPlan<LEN>::T, 24, false)>(a, mode, grid, nthr, smem, s);
 #define HS_ROW_MORE_CASE(LEN)                                                                             \
   case LEN:                                                                                              \
-    if (occ != nullptr) return row_occ_one<float, MODE, LEN>(nthr, smem, occ);                            \
+    if (occ != nullptr) return row_occ_one<float, MODE, LEN, true>(nthr, smem, occ);                      \
     return row_launch<float, MODE, LEN, true>(*a, nb, nthr, smem, s);
 
 // Kernels for plans with a radix-5, 7 or 11 stage, in their own translation unit.

@@ -261,19 +261,11 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
         __syncthreads();  // every group is done with the staged input
         if (act) {
           T* o = reinterpret_cast<T*>(stg) + (size_t)(2 * grp) * n1;
-          if constexpr (LF > 0) {
 #pragma unroll
-            for (int j = 0; j < LF / T8C; ++j) {
-              const C w = z[zfwd(j)];
-              o[t + j * T8C] = w.x;
-              o[n1 + t + j * T8C] = w.y;
-            }
-          } else {
-            for (int x = t; x < n1; x += T8) {
-              const C w = z[zi(x)];
-              o[x] = w.x;
-              o[n1 + x] = w.y;
-            }
+          for (int j = 0; j < LF / T8C; ++j) {
+            const C w = z[zfwd(j)];
+            o[t + j * T8C] = w.x;
+            o[n1 + t + j * T8C] = w.y;
           }
         }
         fence_async_smem();
@@ -326,31 +318,6 @@ __global__ void __launch_bounds__(256, row_min_blocks(sizeof(T) == 8, LF > 0 && 
       } else {
         fft_smem<false, false, (LF < 0)>(reinterpret_cast<C*>(smraw), pitch, 1, 3, G, plan.L, plan.nstage, plan.packed, a.tw,
                                tid, nthr);
-      }
-      if (bulk) {
-        __syncthreads();  // every group is done with the staged input
-        if (act) {
-          C* A = reinterpret_cast<C*>(stg) + (size_t)(2 * grp) * P;
-          C* B = A + P;
-          for (int k = t; k < P; k += T8) {
-            C va = cmk<C>(0, 0), vb = cmk<C>(0, 0);
-            if (k < nh) {
-              const C zk = z[zi(k)];
-              const C zn = z[zi(k == 0 ? 0 : n1 - k)];
-              va = cmk<C>(T(0.5) * (zk.x + zn.x), T(0.5) * (zk.y - zn.y));
-              vb = cmk<C>(T(0.5) * (zk.y + zn.y), T(0.5) * (zn.x - zk.x));
-            }
-            A[k] = va;
-            B[k] = vb;
-          }
-        }
-        fence_async_smem();
-        __syncthreads();
-        if (tid == 0) {
-          bulk_s2g(a.spec_out + 2 * (size_t)b * G * P, stg, (unsigned)(nr * L.outbytes));
-          bulk_commit();
-        }
-        continue;
       }
       group_sync(wsync);
       if (act) {
