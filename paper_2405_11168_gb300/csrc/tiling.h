@@ -63,9 +63,12 @@ inline double pick_zchunk64(int yt, int n3, int ty, int warps, int per_sm, int n
 }
 
 // Planes whose sums a thread of the FP32 real-space pass keeps in FP32 registers before they go to its
-// two-float sums: 4 (at most 16 stress values per chain), fewer on small grids, whose chunks are short and whose
-// passes wait for latency and not for instructions, so that the addition is free there.
-inline int sum_planes(int yt, int n3) { return (int)std::max(1LL, std::min(4LL, (long long)yt * n3 / 1024)); }
+// two-float sums: those of a chunk if the pass had about 1024 blocks, at most 4 (16 stress values per chain).
+// Small grids, whose sums have few terms, keep chains of one plane; their passes wait for latency, not for instructions.
+inline int sum_planes(int yt, int n3) {
+  const int nz = std::min(n3, (1024 + yt - 1) / yt);
+  return std::min(4, (n3 + nz - 1) / nz);
+}
 
 // z chunk of the FP32 real-space pass.  With w warps on an SM a plane of a block takes about 1.15 + 0.1 w
 // (latency, then issue slots), so a chunk costs that for its planes, the recomputed one and a start worth
