@@ -1468,7 +1468,7 @@ static hs_status create_impl(hs_ctx** out, const int grid[3], const hs_material*
   c->ty64 = c->ty;
   c->zc64 = c->zc;
   if (o.precision == HS_FP32_REFINED) {
-    int t = ytile;  // the FP64 sweep's tile follows an explicit ytile, halved while it does not fit
+    int t = o.ytile;  // the FP64 sweep's tile follows an explicit ytile, halved while it does not fit
     while (t > 2 && !tile_fits(t, true)) t /= 2;
     pick64(t, 0, &c->ty64, &c->zc64);
   }
