@@ -7,12 +7,11 @@
 // natural order.  Every stage is done in place: a thread loads all of its
 // butterflies' inputs into registers, the block synchronises, then it writes.
 //
-// Threads per sequence: ceil(L/kE) with kE = 8 elements per thread, so a
-// thread never holds more than ceil(kE/R) butterflies of one stage; radices
-// are 8, 4, 3 and 2 (a radix-16 DFT is available but keeps too many values
-// live for the generic stage loop), and 5, 7 and 11 for the other supported
-// lengths: their length-R DFT is the plain O(R^2) sum with coefficients
-// w_R^{mk} = w_L^{(L/R)(mk mod R)} read from the same twiddle table.  Sequence s, element e lives at
+// Run-time plans: ceil(L/kE) threads per sequence with kE = 8 elements per thread,
+// so a thread never holds more than ceil(kE/R) butterflies of one stage; radices
+// are 8, 4, 3 and 2, and 5, 7 and 11 in kernels of their own.  Compile-time plans
+// (below) choose their threads and take radices up to 16.  Length-5, 7 and 11 DFTs fold the mirrored
+// inputs and use constant coefficients (DftPrime).  Sequence s, element e lives at
 // buf[s*ss + e*es].  Forward = exp(-2 pi i nk/L), inverse = exp(+...), both
 // unnormalised.  Twiddles come from a per-axis table w_L^j = exp(-2 pi i j/L),
 // j < L, computed on the host.
@@ -422,9 +421,11 @@ __host__ __device__ inline bool plan_ext(const FftPlan& p) {
 // 78, 188 (16 x 16: 78, 217); rows 256 as 16 x 16 81 and 73 (8 x 8 x 4: 87, 78), 192 as 4 x 4 x 12 48
 // (8 x 4 x 6: 67; run-time plan 84), 96 as 4 x 4 x 6 10.5 (8 x 12: 11.8), 128 in FP64 as 8 x 4 x 4 158 (8 x 16: 179).
 // ---------------------------------------------------------------------------
-// Lengths with a factor 5, 7 or 11 (FP32): as the run-time plan, whose index arithmetic, predicates and radix
-// switch cost three times the butterflies, a y pass of 112 took 38 us, a z pass of 88 58 and an x pass of
-// 160 37 (160 x 112 x 88).
+// Further FP32 lengths, most with a factor 5, 7 or 11: as the run-time plan, whose index arithmetic, predicates and
+// radix switch cost three times the butterflies, a y pass of 112 took 38 us, a z pass of 88 58 and an x pass of
+// 160 37 (160 x 112 x 88).  The list is a choice and no measured line: lengths up to 240 with a plan of two (240:
+// three) stages of radices up to 16, most of them multiples of 8, at about 1.5 MB of library each.  168, 200,
+// 216, 264, 280, 288, 320 and the lengths between have none and run the run-time plan.
 template <int LEN, int THREADS, int NST, int R0, int R1, int R2 = 1, int R3 = 1> struct FixedPlan {
   static constexpr int L = LEN, n = NST, T = THREADS;
   __host__ __device__ static constexpr int r(int i) { return i == 0 ? R0 : i == 1 ? R1 : i == 2 ? R2 : R3; }

@@ -67,7 +67,7 @@ template <typename T>
 cudaError_t launch_col(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s);
 
 // persistent double-buffered column pass (COL_Y_FWD, COL_Y_INV, COL_Z_GREEN) for the compile-time
-// lengths 64, 128, 256, 512 with the default tile and block size: grid.x persistent blocks,
+// lengths 128, 192, 256, 384, 512 with the default tile and block size: grid.x persistent blocks,
 // grid.z items; cudaErrorNotSupported when no such variant exists
 template <typename T>
 cudaError_t launch_colp(const ColArgs<T>& a, int mode, int ct, dim3 grid, int nthr, size_t smem, cudaStream_t s);

@@ -72,9 +72,10 @@ inline int sum_planes(int yt, int n3) {
 
 // z chunk of the FP32 real-space pass.  With w warps on an SM a plane of a block takes about 1.15 + 0.1 w
 // (latency, then issue slots), so a chunk costs that for its planes, the recomputed one and a start worth
-// 1.3 more, for every full wave of the resident blocks and for what is left over.  Measured at 128^3 (us): chunks 4 / 5 / 8 / 10 / 13 / 16 / 32: 41.9 / 36.8 / 43.0 /
-// 33.9 / 39.0 / 39.1 / 59.5, at 512^3 26 / 37 / 43 / 52 / 64: 1271 / 1240 / 1299 / 1261 / 1228; the model
-// ranks them so.  The shortest chunk within 1% of the best: its sums are the shortest too.
+// 1.3 more, for every full wave of the resident blocks and for what is left over.  Measured at 128^3 (us): chunks
+// 4 / 5 / 8 / 10 / 13 / 16 / 32: 41.9 / 38.4 / 44.2 / 34.7 / 41.3 / 41.4 / 63.7, at 256^3 16 / 24 / 26 / 29 / 32:
+// 177 / 187 / 192 / 176 / 192, at 512^3 26 / 37 / 43 / 52 / 64: 1284 / 1255 / 1313 / 1281 / 1247; the model takes
+// 10, 29 and 40 (1248).  The shortest chunk within 1% of the best: the tail of the last wave is the shortest too.
 inline int pick_zchunk32(int yt, int n3, int warps, int per_sm, int nsm) {
   std::vector<double> cost(std::min(n3, 64) + 1, 0.0);
   double best = 1e300;
